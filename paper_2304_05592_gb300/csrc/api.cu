@@ -5,8 +5,10 @@
 
 #include <algorithm>
 #include <functional>
+#include <memory>
 #include <mutex>
 
+#include "chip.h"
 #include "internal.h"
 
 using namespace wave;
@@ -72,9 +74,11 @@ struct Layout {
     float* slots_src = nullptr;
     float* dsyn = nullptr;
     float* dmv = nullptr;
+    float* tacc = nullptr;  // on-chip adjoint: the receivers' share of the imaging sums
     __nv_bfloat16* st16 = nullptr;
     size_t bytes = 0;
     StepMaps maps;
+    ChipPlan cf, ca;  // the on-chip time loop's split for forward / adjoint steps (C = 0: not used)
 
     size_t field() const { return (size_t)nshot * d.cell; }
     float* buf(int i) const { return pool + (size_t)i * field(); }
@@ -188,6 +192,7 @@ wave_status_t plan(const wave_grid_t* g, int op, int nshot, int nsrc, const floa
     if (op == 1) L.slots_src = c.take<float>(nt * L.hs.idx.size());
     if (op == 2) {
         L.dsyn = c.take<float>((size_t)nshot * nt * nrec);
+        if (d.ndim == 2) L.tacc = c.take<float>(L.hr.idx.size());
         if (store == WAVE_STORE_BF16) L.st16 = c.take<__nv_bfloat16>(nt * L.field());
     }
     L.bytes = c.off;
@@ -260,6 +265,7 @@ wave_status_t make_maps(Layout& L)
                                                                                                 : WAVE_ERR_CUDA;
     }
     if (d.ndim != 2) return WAVE_OK;
+    if ((L.op == 0 && L.cf.C) || (L.op == 1 && L.ca.C) || (L.op == 2 && L.cf.C && L.ca.C)) return WAVE_OK;
     const cuuint64_t fdims[4] = {(cuuint64_t)d.Nx, (cuuint64_t)d.Nz, (cuuint64_t)L.nshot, (cuuint64_t)L.nbuf};
     const cuuint64_t fstr[3] = {(cuuint64_t)d.P * 4, (cuuint64_t)d.cell * 4, (cuuint64_t)L.field() * 4};
     const cuuint64_t kdims[2] = {(cuuint64_t)d.Nx, (cuuint64_t)d.Nz};
@@ -427,6 +433,42 @@ float sponge_coefficient(const Dims& d)
     return (float)(3.0 * log(1000.0) * d.h / (4.0 * d.dt * d.vref * nb * nb * nb));
 }
 
+// Time of one step of all shots with a launch per step (us), to weigh against
+// the on-chip loop's estimate.  Measured with the default kernels: 4.15 / 4.7 us
+// for one shot (no faster than launches queue), 1.95 / 2.85 us more for each of
+// the up to 4 shots a CTA works through (9.6 / 13.6 us at 4 shots of 480 x 280,
+// 11.0 / 14.1 us at 16 of 336 x 208), then the tile kernels' rate (16.6 / 20 us
+// at 32 shots of 592 x 336).
+float launched_step_us(const Dims& d, int nshot, bool adjoint)
+{
+    const float pts = (float)d.Nz * d.Nx * nshot, g = (float)std::min(nshot, 4);
+    return adjoint ? std::max({4.7f, 2.2f + 2.85f * g, 3.1e-6f * pts}) : std::max({4.15f, 2.0f + 1.95f * g, 2.55e-6f * pts});
+}
+
+// Decides between the on-chip time loop and the per-step kernels, per
+// direction: a forced or tuned variant is followed where the loop can take the
+// problem, otherwise the faster estimate wins.
+void choose_chip(Layout& L)
+{
+    if (L.d.ndim != 2 || L.op == 3) return;
+    auto pick = [&](int which, int& v, bool set, int mode, const HostTaps& inj, const HostTaps& gat) {
+        const bool asked = variant_info(which, v).kind == 8;
+        ChipPlan p;
+        if (asked || !set) p = chip_plan(L.d, L.t, L.nshot, mode, inj, gat);
+        // (the estimates are good to 10 %; where they nearly meet the launches have the better of it)
+        if (p.C && !asked && 1.15f * p.step_us >= launched_step_us(L.d, L.nshot, which == 1)) p.C = 0;
+        if (L.nbuf >= 32768) p.C = 0;  // buffer indices travel as 16-bit numbers
+        if (p.C) v = chip_variant(which);
+        else if (asked) v = default_variant(which);
+        return p;
+    };
+    const HostTaps none;
+    if (L.op == 0 || L.op == 2) L.cf = pick(0, L.t.vf, L.t.set_f, L.st16 ? kChipFwdBF16 : kChipForward, L.hs, L.hr);
+    if (L.op == 1) L.ca = pick(1, L.t.va, L.t.set_a, kChipAdjoint, L.hr, L.hs);
+    if (L.op == 2)
+        L.ca = pick(1, L.t.va, L.t.set_a, L.store == WAVE_STORE_BF16 ? kChipAdjBF16 : kChipAdjF32, L.hr, none);
+}
+
 // Uploads tables, prepares the model, queues its validation (non-finite
 // velocities and the stability limit set bits of the device error word; the
 // host does not wait for them), fills the injection factors and encodes the
@@ -446,6 +488,7 @@ wave_status_t setup(Layout& L, const float* vel, cudaStream_t s)
     // Adjoint receiver injection adds w r / (m + e) = kap (h/dt)^2 w r / (1 + eps).
     launch_tapfac(L.d, L.tr.l, L.kap, (float)(h * h / (dt * dt)), ceps, s);
     CK(cudaGetLastError());
+    choose_chip(L);
     return make_maps(L);
 }
 
@@ -541,6 +584,136 @@ void adj_step(const Layout& L, int cur, int prev, int k, const float* amp_a, con
     launch_step(L.t, L.d.ndim, true, a, &L.maps, s);
 }
 
+// Time steps in the order the executor asks for them.  With a launch per step
+// they go to fwd_step / adj_step as they come; with the on-chip loop,
+// consecutive steps that continue one state gather into one launch, queued by
+// flush() (the caller flushes before it queues work that reads their results).
+class StepQueue {
+public:
+    StepQueue(const Layout& l, const float* wavelet, const float* amp_a, const float* amp_b, bool gather_src,
+              cudaStream_t stream)
+        : L(l), wavelet_(wavelet), amp_a_(amp_a), amp_b_(amp_b), gather_src_(gather_src), s(stream)
+    {
+        if (L.cf.C || L.ca.C) a_.reset(new ChipArgs);
+    }
+
+    // u^{n+1} into buffer out; st16: store row n + 1; t32: FP32 store buffer (-1: none).
+    // keep: the level is read later (a checkpoint, or the state an adjoint step or a later run starts from).
+    void fwd(int cur, int prev, int out, int n, bool record, __nv_bfloat16* st16, int t32, bool keep)
+    {
+        if (!L.cf.C) {
+            flush();
+            fwd_step(L, cur, prev, out, n, wavelet_, record, st16, t32 >= 0 ? L.buf(t32) : nullptr, s);
+            return;
+        }
+        if (dir_ != 1 || out_ != cur || n != a_->first + a_->nsteps ||
+            (a_->keep_mode == kKeepTable && a_->nsteps == kChipTable)) {
+            flush();
+            begin(1, cur, prev, n);
+            a_->keep_mode = t32 >= 0 ? kKeepRows : (keep ? kKeepTable : kKeepNone);
+            a_->row0 = t32 - (n + 1);
+            a_->st16 = L.st16 && st16 ? L.st16 : nullptr;
+            a_->rec_from = 1 << 30;
+        }
+        if (record && a_->rec_from > n) a_->rec_from = n;
+        if (a_->keep_mode == kKeepTable) a_->tab[a_->nsteps] = out >= L.iS0 ? (short)out : (short)-1;
+        push(out, a_->keep_mode == kKeepTable);
+    }
+
+    // mu^k over mu^{k+2} (buffer prev); uf: buffer of u^k, or row uf16 of the BF16 store (-1: none).
+    void adj(int cur, int prev, int k, int uf, int uf16)
+    {
+        if (!L.ca.C) {
+            flush();
+            adj_step(L, cur, prev, k, amp_a_, amp_b_, gather_src_, uf, uf16, s);
+            return;
+        }
+        if (dir_ != 2 || out_ != cur || k != a_->first - a_->nsteps || (uf >= 0 && a_->nsteps == kChipTable)) {
+            flush();
+            begin(2, cur, prev, k);
+            a_->uf16 = uf16 >= 0 ? L.st16 : nullptr;
+            a_->g_buf = L.iG;
+            if (L.op == 2) a_->tacc = L.tacc;
+        }
+        if (uf >= 0) a_->tab[a_->nsteps] = (short)uf;
+        push(prev, true);
+    }
+
+    // Queues the gathered steps.
+    void flush()
+    {
+        if (dir_ == 0) return;
+        const cudaError_t e = launch_chip(dir_ == 1 ? L.cf : L.ca, *a_, L.nshot, s);
+        if (e != cudaSuccess) {
+            note_cuda_error(e);
+            failed_ = true;
+        }
+        dir_ = 0;
+    }
+    bool failed() const { return failed_; }
+
+private:
+    void begin(int dir, int cur, int prev, int first)
+    {
+        const Dims& d = L.d;
+        ChipArgs& a = *a_;
+        dir_ = dir;
+        a.kap = L.kap;
+        a.pool = L.pool;
+        a.field = (long long)L.field();
+        a.cell = d.cell;
+        a.Nx = d.Nx;
+        a.Nz = d.Nz;
+        a.P = d.P;
+        a.nb = d.nb;
+        a.nx = d.nx;
+        a.nz = d.nz;
+        a.ceps = sponge_coefficient(d);
+        a.first = first;
+        a.nsteps = 0;
+        a.cur = cur;
+        a.prev = prev;
+        a.out_last = a.out_prev = -1;
+        a.keep_mode = kKeepNone;
+        a.row0 = 0;
+        a.st16 = nullptr;
+        a.uf16 = nullptr;
+        a.g_buf = -1;
+        a.tacc = nullptr;
+        a.inj = a.gat = TapList();
+        a.amp_a = a.amp_b = nullptr;
+        a.slots = nullptr;
+        a.rec_from = 0;
+        a.cps = L.t.cells_per_shot();
+        a.err = L.err;
+        const bool f = dir == 1;
+        if (f ? L.nsrc > 0 && L.ts.l.ntap > 0 : L.nrec > 0 && L.tr.l.ntap > 0) {
+            a.inj = f ? L.ts.l : L.tr.l;
+            a.amp_a = f ? wavelet_ : amp_a_;
+            a.amp_b = f ? nullptr : amp_b_;
+        }
+        if (f ? L.slots_rec && L.nrec > 0 && L.tr.l.ntap > 0 : gather_src_ && L.nsrc > 0 && L.ts.l.ntap > 0) {
+            a.gat = f ? L.tr.l : L.ts.l;
+            a.slots = f ? L.slots_rec : L.slots_src;
+        }
+    }
+    void push(int out, bool keep)
+    {
+        a_->out_prev = a_->out_last;
+        a_->out_last = keep ? out : -1;
+        out_ = out;
+        ++a_->nsteps;
+    }
+
+    const Layout& L;
+    const float *wavelet_, *amp_a_, *amp_b_;
+    bool gather_src_;
+    cudaStream_t s;
+    std::unique_ptr<ChipArgs> a_;
+    int dir_ = 0, out_ = -1;  // direction of the gathered steps (0: none), buffer of their last level
+    bool failed_ = false;
+};
+
 wave_status_t check_work(const Layout& L, void* work, size_t work_bytes)
 {
     if (L.bytes > 0 && (!work || work_bytes < L.bytes)) return WAVE_ERR_WORKSPACE;
@@ -590,8 +763,8 @@ wave_status_t queued()
 // only renames which buffers hold (u^j, u^{j-1}), the last two steps of an
 // advance that ends in a save write straight into the slot, and a step that
 // starts from a slot writes out of place into W0/W1.
-wave_status_t run_checkpointed(Layout& L, const float* wavelet, const float* amp_a, const float* amp_b,
-                               bool record_data, const std::function<void()>& finalize_data, cudaStream_t s)
+wave_status_t run_checkpointed(Layout& L, StepQueue& q, bool record_data, const std::function<void()>& finalize_data,
+                               cudaStream_t s)
 {
     const Dims& d = L.d;
     const Schedule sch = make_schedule(d.nt, L.nsnap);
@@ -615,7 +788,7 @@ wave_status_t run_checkpointed(Layout& L, const float* wavelet, const float* amp
                 else if (prev == W0 || prev == W1) out = prev;
                 else out = cur == W0 ? W1 : W0;
                 const bool rec = record_data && n >= recorded;
-                fwd_step(L, cur, prev, out, n, wavelet, rec, nullptr, nullptr, s);
+                q.fwd(cur, prev, out, n, rec, nullptr, -1, true);
                 if (rec) recorded = n + 1;
                 prev = cur;
                 cur = out;
@@ -625,6 +798,8 @@ wave_status_t run_checkpointed(Layout& L, const float* wavelet, const float* amp
         }
         case kSave: {
             const int k = act.a;
+            // the zero batch can be copied ahead of gathered steps, anything else waits for them
+            if ((cur != slot_cur(k) && cur != Z) || (prev != slot_prev(k) && prev != Z)) q.flush();
             if (cur != slot_cur(k)) CK(cudaMemcpyAsync(L.buf(slot_cur(k)), L.buf(cur), fb, cudaMemcpyDeviceToDevice, s));
             if (prev != slot_prev(k))
                 CK(cudaMemcpyAsync(L.buf(slot_prev(k)), L.buf(prev), fb, cudaMemcpyDeviceToDevice, s));
@@ -643,15 +818,16 @@ wave_status_t run_checkpointed(Layout& L, const float* wavelet, const float* amp
             break;
         case kFinalize:
             if (record_data && recorded != sch.K) return WAVE_ERR_ARG;  // not reachable
+            q.flush();
             finalize_data();
             break;
         case kAdjointPair: {
             const int j = sch.state_of(act.a);
             if (j != state) return WAVE_ERR_ARG;  // not reachable
-            adj_step(L, A0 + acur, A0 + 1 - acur, j, amp_a, amp_b, false, cur, -1, s);
+            q.adj(A0 + acur, A0 + 1 - acur, j, cur, -1);
             acur ^= 1;
             if (j - 1 >= 1) {
-                adj_step(L, A0 + acur, A0 + 1 - acur, j - 1, amp_a, amp_b, false, prev, -1, s);
+                q.adj(A0 + acur, A0 + 1 - acur, j - 1, prev, -1);
                 acur ^= 1;
             }
             break;
@@ -722,10 +898,13 @@ wave_status_t wave_forward(const wave_grid_t* grid, const float* vel, int nshot,
     const size_t nrow = L.hr.idx.size();
     if (nrow) CK(cudaMemsetAsync(L.slots_rec, 0, nrow * sizeof(float), s));
     int cur = 0;
+    StepQueue q(L, wavelet, nullptr, nullptr, false, s);
     for (int n = 0; n + 1 < L.d.nt; ++n) {
-        fwd_step(L, cur, 1 - cur, 1 - cur, n, wavelet, true, nullptr, nullptr, s);
+        q.fwd(cur, 1 - cur, 1 - cur, n, true, nullptr, -1, false);
         cur ^= 1;
     }
+    q.flush();
+    if (q.failed()) return WAVE_ERR_CUDA;
     if (nrec) {
         launch_finalize(L.tr.l, L.slots_rec, nshot, L.d.nt, data, s);
         launch_nan_scan(data, (long long)nshot * L.d.nt * nrec, L.err, s);
@@ -750,10 +929,13 @@ wave_status_t wave_adjoint(const wave_grid_t* grid, const float* vel, int nshot,
     const size_t nrow = L.hs.idx.size();
     if (nrow) CK(cudaMemsetAsync(L.slots_src + (size_t)(L.d.nt - 1) * nrow, 0, nrow * sizeof(float), s));
     int cur = 0;
+    StepQueue q(L, nullptr, resid, nullptr, true, s);
     for (int k = L.d.nt - 1; k >= 1; --k) {
-        adj_step(L, cur, 1 - cur, k, resid, nullptr, true, -1, -1, s);
+        q.adj(cur, 1 - cur, k, -1, -1);
         cur ^= 1;
     }
+    q.flush();
+    if (q.failed()) return WAVE_ERR_CUDA;
     if (nsrc) {
         launch_finalize(L.ts.l, L.slots_src, nshot, L.d.nt, src_out, s);
         launch_nan_scan(src_out, (long long)nshot * L.d.nt * nsrc, L.err, s);
@@ -794,6 +976,7 @@ wave_status_t gradient_impl(const wave_grid_t* grid, const float* vel, int nshot
     CK(cudaMemsetAsync(L.buf(0), 0, 6 * fb, s));
     const size_t nrow = L.hr.idx.size();
     if (nrow && !given) CK(cudaMemsetAsync(L.slots_rec, 0, nrow * sizeof(float), s));
+    if (L.ca.C && !L.ca.add_rows && nrow) CK(cudaMemsetAsync(L.tacc, 0, nrow * sizeof(float), s));
     const long long ndata = (long long)nshot * d.nt * nrec;
     const int K = d.nt - 1;
     const float* amp_a = given ? resid : L.dsyn;
@@ -810,29 +993,33 @@ wave_status_t gradient_impl(const wave_grid_t* grid, const float* vel, int nshot
     };
 
     const int W0 = L.iW0, A0 = L.iA0;
+    StepQueue q(L, wavelet, amp_a, amp_b, false, s);
     if (store != WAVE_STORE_CHECKPOINT) {
         if (L.st16) CK(cudaMemsetAsync(L.st16, 0, field * sizeof(__nv_bfloat16), s));
         if (L.iT0 >= 0) CK(cudaMemsetAsync(L.buf(L.iT0), 0, fb, s));
         int cur = 0;
         for (int n = 0; n < K; ++n) {
             __nv_bfloat16* r16 = L.st16 ? L.st16 + (size_t)(n + 1) * field : nullptr;
-            float* r32 = L.iT0 >= 0 ? L.buf(L.iT0 + n + 1) : nullptr;
-            fwd_step(L, W0 + cur, W0 + 1 - cur, W0 + 1 - cur, n, wavelet, !given, r16, r32, s);
+            q.fwd(W0 + cur, W0 + 1 - cur, W0 + 1 - cur, n, !given, r16, L.iT0 >= 0 ? L.iT0 + n + 1 : -1, false);
             cur ^= 1;
         }
+        q.flush();
         finalize_data();
         int acur = 0;
         for (int k = K; k >= 1; --k) {
-            if (L.st16) adj_step(L, A0 + acur, A0 + 1 - acur, k, amp_a, amp_b, false, -1, k, s);
-            else adj_step(L, A0 + acur, A0 + 1 - acur, k, amp_a, amp_b, false, L.iT0 + k, -1, s);
+            q.adj(A0 + acur, A0 + 1 - acur, k, L.st16 ? -1 : L.iT0 + k, L.st16 ? k : -1);
             acur ^= 1;
         }
+        q.flush();
     } else if (K < 1) {
         finalize_data();
     } else {
-        st = run_checkpointed(L, wavelet, amp_a, amp_b, !given, finalize_data, s);
+        st = run_checkpointed(L, q, !given, finalize_data, s);
         if (st) return st;
+        q.flush();
     }
+    if (q.failed()) return WAVE_ERR_CUDA;
+    if (L.ca.C && !L.ca.add_rows) launch_chip_tap_gradient(L.tr.l, d.nt, d.cell, L.tacc, L.buf(L.iG), s);
     // A0 and A1 (contiguous) are free now: scratch for the reduction.
     launch_grad_reduce(d, L.buf(L.iG), gradient_accumulators(L.t, d.ndim, nshot), L.buf(A0), grad,
                        wrt == WAVE_WRT_VELOCITY ? vel : nullptr, s);
@@ -960,12 +1147,36 @@ wave_status_t wave_autotune(const wave_grid_t* grid, const float* vel, int nshot
     const int nstep = std::max(1, std::min(steps, L.d.nt - 1));
     float best[2] = {1e30f, 1e30f};
     int pick[2] = {current_variant(0), current_variant(1)};
+    L.cf = L.ca = ChipPlan();
+    const HostTaps none;
     for (int which = 0; which < 2; ++which) {
         for (int v = 0; v < variant_count(which); ++v) {
             if (which == 0) L.t.vf = v;
             else L.t.va = v;
+            int m = nstep;
+            if (variant_info(which, v).kind == 8) {
+                // the on-chip loop loads its state once per run, and runs are long: timed over more steps
+                ChipPlan& p = which == 0 ? L.cf : L.ca;
+                p = which == 0 ? chip_plan(L.d, L.t, nshot, kChipForward, L.hs, L.hr)
+                               : chip_plan(L.d, L.t, nshot, kChipAdjF32, L.hr, none);
+                if (!p.C || L.d.nt < 2) {
+                    p.C = 0;
+                    continue;
+                }
+                m = std::max(1, std::min(16 * nstep, L.d.nt - 1));
+            }
             if (make_maps(L)) continue;
             auto run = [&](int n_steps) {
+                if (L.cf.C || L.ca.C) {
+                    StepQueue q(L, wavelet, L.dsyn, nullptr, false, s);
+                    for (int k = 0; k < n_steps; ++k) {
+                        const int b = k & 1;
+                        if (which == 0) q.fwd(L.iW0 + b, L.iW0 + 1 - b, L.iW0 + 1 - b, k, true, nullptr, -1, false);
+                        else q.adj(L.iA0 + b, L.iA0 + 1 - b, L.d.nt - 1 - k, L.iW0, -1);
+                    }
+                    q.flush();
+                    return;
+                }
                 for (int k = 0; k < n_steps; ++k) {
                     const int n = k % std::max(1, L.d.nt - 1);
                     if (which == 0) fwd_step(L, L.iW0 + (k & 1), L.iW0 + 1 - (k & 1), L.iW0 + 1 - (k & 1), n, wavelet,
@@ -974,9 +1185,9 @@ wave_status_t wave_autotune(const wave_grid_t* grid, const float* vel, int nshot
                                   L.iW0, -1, s);
                 }
             };
-            run(2);
+            run(std::min(2, m));
             cudaEventRecord(e0, s);
-            run(nstep);
+            run(m);
             cudaEventRecord(e1, s);
             if (cudaEventSynchronize(e1) != cudaSuccess) {
                 cudaEventDestroy(e0);
@@ -986,6 +1197,8 @@ wave_status_t wave_autotune(const wave_grid_t* grid, const float* vel, int nshot
             }
             float ms = 0.0f;
             cudaEventElapsedTime(&ms, e0, e1);
+            ms *= (float)nstep / m;
+            L.cf = L.ca = ChipPlan();
             if (ms < best[which]) {
                 best[which] = ms;
                 pick[which] = v;

@@ -49,6 +49,7 @@ struct Tiling {
     int ncx, ncy, ncz;
     int vf, va;  // 2D kernel variants for the forward / adjoint steps
     int v3;      // 3D kernel variant
+    bool set_f = false, set_a = false;  // vf / va were forced or tuned, not defaulted
     long long cells_per_shot() const { return (long long)ncx * ncy * ncz; }
 };
 
@@ -154,7 +155,8 @@ constexpr int kTZc2 = 8;          // 2D tap-cell height: divides every 2D tile h
 // in shared memory instead of registers, bit 2: the adjoint's forward level
 // comes by TMA too, bits 3 / 4: a 3- / 4-stage ring instead of 2), or
 // the persistent kernel over (tile, shot) items (kind 5, R = thread rows), or
-// the z-window kernel (kind 7, below).
+// the z-window kernel (kind 7, below), or the on-chip time loop (kind 8,
+// chip.h: many steps per launch, one gradient accumulator per shot).
 // With kinds 2 and 4 in the adjoint, the gradient buffer holds one
 // accumulator per shot group; with kind 5, one per CTA segment of a tile.
 struct Variant2D {
@@ -172,6 +174,8 @@ Variant2D variant_info(int which, int v);
 int current_variant(int which);           // the selected or default variant
 int select_variant(int which, int v);     // v = -1 restores the default; 0 on success
 bool variant_forced(int which);           // true after wave_set_variant(which, v >= 0)
+int default_variant(int which);
+int chip_variant(int which);              // the kind-8 entry of the 2D tables
 
 // Remembers the last failing CUDA call of this thread (profile.cu).
 void note_cuda_error(cudaError_t e);
@@ -181,7 +185,8 @@ void note_cuda_error(cudaError_t e);
 // sampled launches in a pair of CUDA events on the launching stream.
 void count_launch(int n = 1);
 void count_step_launch();  // a stencil time step (launch_step)
-bool profile_sample(bool adjoint, cudaStream_t s, cudaEvent_t* stop);
+// steps: time steps the launch makes (samples are reported per step)
+bool profile_sample(bool adjoint, cudaStream_t s, cudaEvent_t* stop, int steps = 1);
 void profile_close(cudaEvent_t stop, cudaStream_t s);
 
 // Tiling choice (plan.cu): the 2D variants come from wave_set_variant, else

@@ -1742,7 +1742,7 @@ static const Variant2D kFwd2D[] = {{0, 32, 4, 0, 0}, {1, 48, 6, 2, 0}, {1, 32, 4
                                    {4, 16, 8, 2, 4},  {7, 16, 4, 0, 2}, {7, 16, 4, 1, 4}, {7, 16, 2, 2, 2},
                                    {7, 32, 8, 3, 2},  {7, 32, 4, 4, 2}, {7, 16, 8, 5, 2}, {4, 16, 8, 9, 2},
                                    {4, 16, 8, 9, 4},  {4, 16, 8, 17, 4}, {4, 16, 8, 9, 8}, {4, 16, 8, 17, 8}, {4, 16, 8, 41, 4},
-                                   {4, 16, 8, 33, 2},  {4, 16, 8, 41, 8}, {4, 16, 8, 49, 4}};
+                                   {4, 16, 8, 33, 2},  {4, 16, 8, 41, 8}, {4, 16, 8, 49, 4}, {8, 16, 8, 0, 0}};
 static const Variant2D kAdj2D[] = {{0, 32, 4, 0, 0}, {1, 24, 3, 3, 0}, {1, 16, 2, 4, 0}, {1, 32, 4, 2, 0},
                                    {2, 32, 8, 0, 4}, {2, 16, 8, 0, 4}, {2, 32, 8, 0, 8}, {2, 16, 8, 0, 2},
                                    {3, 24, 4, 1, 0}, {3, 24, 4, 2, 0}, {3, 48, 4, 2, 0}, {3, 16, 8, 2, 0},
@@ -1754,7 +1754,7 @@ static const Variant2D kAdj2D[] = {{0, 32, 4, 0, 0}, {1, 24, 3, 3, 0}, {1, 16, 2
                                    {7, 16, 4, 1, 4}, {7, 16, 2, 2, 2}, {7, 32, 8, 3, 2},  {7, 32, 4, 4, 2},
                                    {7, 16, 8, 5, 2}, {4, 16, 8, 5, 2}, {4, 16, 8, 13, 2}, {4, 16, 8, 13, 4},
                                    {4, 16, 8, 5, 4}, {4, 16, 8, 69, 4}, {4, 16, 8, 101, 4}, {4, 16, 8, 37, 4},
-                                   {4, 16, 8, 101, 8}, {4, 16, 8, 45, 4}, {4, 16, 8, 101, 2}};
+                                   {4, 16, 8, 101, 8}, {4, 16, 8, 45, 4}, {4, 16, 8, 101, 2}, {8, 16, 8, 0, 0}};
 // 3D variants (which = 2; TZ = planes per CTA, R = tile rows in y, NST = ring
 // slots, G = 1 for the ring without block barriers, G = PF + 1 for the ring
 // whose model and previous level arrive PF planes ahead by cp.async): kind 0
@@ -1788,6 +1788,10 @@ int current_variant(int which)
     if (which < 0 || which > 2) return -1;
     return g_selected[which] >= 0 ? g_selected[which] : kDefaultVariant[which];
 }
+
+int default_variant(int which) { return kDefaultVariant[which]; }
+
+int chip_variant(int which) { return variant_count(which) - 1; }
 
 bool variant_forced(int which) { return which >= 0 && which <= 2 && g_selected[which] >= 0; }
 

@@ -54,12 +54,15 @@ Tiling choose_tiling(const Dims& d, int nshot)
         t.TZc = kTZc2;
         t.vf = current_variant(0);
         t.va = current_variant(1);
+        t.set_f = variant_forced(0);
+        t.set_a = variant_forced(1);
         // an explicit wave_set_variant wins over a tuned choice
         std::lock_guard<std::mutex> lock(g_tuned_mu);
         auto it = g_tuned.find(std::make_tuple(d.Nx, d.Nz, nshot));
         if (it != g_tuned.end()) {
             if (!variant_forced(0)) t.vf = it->second.first;
             if (!variant_forced(1)) t.va = it->second.second;
+            t.set_f = t.set_a = true;
         }
     } else {
         t.TY = 8;

@@ -13,7 +13,7 @@ namespace {
 struct Sample {
     cudaEvent_t start, stop;
     bool adjoint;
-    long long launches;  // step launches the sample covers
+    long long launches;  // time steps the sample covers
 };
 
 std::atomic<long long> g_launches{0};
@@ -73,13 +73,13 @@ void count_launch(int n)
 
 void count_step_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 
-bool profile_sample(bool adjoint, cudaStream_t s, cudaEvent_t* stop)
+bool profile_sample(bool adjoint, cudaStream_t s, cudaEvent_t* stop, int steps)
 {
     std::lock_guard<std::mutex> lock(g_mu);
     if (!g_on) return false;
     if (g_runs) {
         if (g_open && g_samples.back().adjoint == adjoint && g_run_stream == s) {
-            ++g_samples.back().launches;
+            g_samples.back().launches += steps;
             return false;
         }
         close_run();
@@ -88,7 +88,7 @@ bool profile_sample(bool adjoint, cudaStream_t s, cudaEvent_t* stop)
         smp.start = take_event();
         smp.stop = take_event();
         smp.adjoint = adjoint;
-        smp.launches = 1;
+        smp.launches = steps;
         if (!smp.start || !smp.stop) return false;
         cudaEventRecord(smp.start, s);
         g_samples.push_back(smp);
@@ -102,7 +102,7 @@ bool profile_sample(bool adjoint, cudaStream_t s, cudaEvent_t* stop)
     smp.start = take_event();
     smp.stop = take_event();
     smp.adjoint = adjoint;
-    smp.launches = 1;
+    smp.launches = steps;
     if (!smp.start || !smp.stop) return false;
     cudaEventRecord(smp.start, s);
     g_samples.push_back(smp);
