@@ -100,7 +100,7 @@ wave_status_t check_grid(const wave_grid_t* g)
 
 void carve_taps(Carver& c, const HostTaps& h, long long ncells_all, DevTaps& t)
 {
-    const size_t ntap = h.idx.size();
+    const size_t ntap = h.ntap;
     t.cell_start = c.take<int>(ncells_all + 1);
     t.idx = c.take<int>(ntap);
     t.fac = c.take<float>(ntap);
@@ -108,7 +108,7 @@ void carve_taps(Carver& c, const HostTaps& h, long long ncells_all, DevTaps& t)
     t.ab = c.take<int>(ntap);
     t.slot = c.take<int>(ntap);
     t.w = c.take<float>(ntap);
-    t.pt_start = c.take<int>(h.pt_start.size());
+    t.pt_start = c.take<int>(h.npt_start);
     t.l.cell_start = t.cell_start;
     t.l.idx = t.idx;
     t.l.fac = t.fac;
@@ -147,9 +147,10 @@ wave_status_t plan(const wave_grid_t* g, int op, int nshot, int nsrc, const floa
     L.nrec = nrec;
     L.store = store;
     const Dims& d = L.d;
-    st = build_taps(d, L.t, nshot, nsrc, src_xyz, L.hs);
+    const bool size_only = base == nullptr;  // (a call that runs has a workspace; without one check_work refuses it)
+    st = build_taps(d, L.t, nshot, nsrc, src_xyz, size_only, L.hs);
     if (st) return st;
-    st = build_taps(d, L.t, nshot, nrec, rec_xyz, L.hr);
+    st = build_taps(d, L.t, nshot, nrec, rec_xyz, size_only, L.hr);
     if (st) return st;
 
     const long long ncells_all = (long long)nshot * L.t.cells_per_shot();
@@ -187,15 +188,16 @@ wave_status_t plan(const wave_grid_t* g, int op, int nshot, int nsrc, const floa
     carve_taps(c, L.hs, ncells_all, L.ts);
     carve_taps(c, L.hr, ncells_all, L.tr);
     L.pool = c.take<float>((size_t)L.nbuf * L.field());
-    if (op == 0 || op == 2 || op == 3) L.slots_rec = c.take<float>(nt * L.hr.idx.size());
+    if (op == 0 || op == 2 || op == 3) L.slots_rec = c.take<float>(nt * L.hr.ntap);
     if (op == 3) L.dmv = c.take<float>(d.cell);
-    if (op == 1) L.slots_src = c.take<float>(nt * L.hs.idx.size());
+    if (op == 1) L.slots_src = c.take<float>(nt * L.hs.ntap);
     if (op == 2) {
         L.dsyn = c.take<float>((size_t)nshot * nt * nrec);
-        if (d.ndim == 2) L.tacc = c.take<float>(L.hr.idx.size());
+        if (d.ndim == 2) L.tacc = c.take<float>(L.hr.ntap);
         if (store == WAVE_STORE_BF16) L.st16 = c.take<__nv_bfloat16>(nt * L.field());
     }
     L.bytes = c.off;
+    if (size_only) return WAVE_OK;
     // Gather weights: receivers sample with w; the source-side adjoint
     // gathers dt^2 w / h^ndim (the transpose of the injection).
     const double hd = d.ndim == 3 ? (double)d.h * d.h * d.h : (double)d.h * d.h;

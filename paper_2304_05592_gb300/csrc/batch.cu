@@ -760,9 +760,9 @@ wave_status_t plan_batch(const wave_problem_t* probs, int nprob, int store, void
         h.t.ncy = 1;
         h.t.ncz = (h.d.Nz + kTZc2 - 1) / kTZc2;
         h.t.vf = h.t.va = 0;
-        wave_status_t st = build_taps(h.d, h.t, 1, q.nsrc, q.src_xyz, h.hs);
+        wave_status_t st = build_taps(h.d, h.t, 1, q.nsrc, q.src_xyz, false, h.hs);
         if (st) return st;
-        st = build_taps(h.d, h.t, 1, q.nrec, q.rec_xyz, h.hr);
+        st = build_taps(h.d, h.t, 1, q.nrec, q.rec_xyz, false, h.hr);
         if (st) return st;
         B.ntile_cap += ((h.d.Nz + kMinTZ - 1) / kMinTZ) * h.t.ncx;
         B.maxnt = std::max(B.maxnt, q.grid.nt);

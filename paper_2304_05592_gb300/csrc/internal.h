@@ -72,11 +72,13 @@ struct HostTaps {
     std::vector<int> cell_start, idx, ab, slot, pt_start;
     std::vector<float> w;
     int npts = 0;
+    size_t ntap = 0, npt_start = 0;  // sizes of the tables, also when only counted
 };
 
 // Builds taps for nshot * npts points; WAVE_ERR_GEOMETRY for a point outside
-// the physical grid.
-wave_status_t build_taps(const Dims& d, const Tiling& t, int nshot, int npts, const float* xyz, HostTaps& out);
+// the physical grid.  count_only: the sizes, not the tables.
+wave_status_t build_taps(const Dims& d, const Tiling& t, int nshot, int npts, const float* xyz, bool count_only,
+                         HostTaps& out);
 
 // TMA descriptors.  Every field batch ([nshot][Nz][P]) of a call lives in one
 // pool of equally sized buffers, so one 4D map addresses any of them through a

@@ -87,30 +87,24 @@ int gradient_accumulators(const Tiling& t, int ndim, int nshot)
 }
 
 // Interpolation taps of one point: bilinear (2D) / trilinear (3D) weights on
-// the padded grid, dropping taps of weight zero.
-static bool point_taps(const Dims& d, const float* c, int* idx, float* w, int* n)
+// the padded grid, dropping taps of weight zero; x, y, z: their grid indices.
+struct PointTap {
+    int x, y, z;
+    float w;
+};
+
+static bool point_taps(const Dims& d, const float* c, PointTap* tap, int* n)
 {
     const int nax = d.ndim;
-    int nphys[3], npad[3];
-    nphys[0] = d.nx;
-    npad[0] = d.Nx;
-    if (nax == 2) {
-        nphys[1] = d.nz;
-        npad[1] = d.Nz;
-    } else {
-        nphys[1] = d.ny;
-        npad[1] = d.Ny;
-        nphys[2] = d.nz;
-        npad[2] = d.Nz;
-    }
-    int i0[3];
+    const int nphys[3] = {d.nx, nax == 2 ? d.nz : d.ny, d.nz}, npad[3] = {d.Nx, nax == 2 ? d.Nz : d.Ny, d.Nz};
+    int i0[3] = {0, 0, 0};
     double fr[3];
     const double h = d.h;
     for (int a = 0; a < nax; ++a) {
         const double x = c[a];
-        if (!std::isfinite(x) || x < 0.0 || x > (nphys[a] - 1) * h) return false;
+        if (!(x >= 0.0 && x <= (nphys[a] - 1) * h)) return false;  // also rejects NaN
         const double f = x / h + d.nb;
-        int i = (int)floor(f);
+        int i = (int)f;  // f >= 0: the floor
         if (i > npad[a] - 2) i = npad[a] - 2;
         i0[a] = i;
         fr[a] = f - i;
@@ -118,84 +112,89 @@ static bool point_taps(const Dims& d, const float* c, int* idx, float* w, int* n
     int k = 0;
     for (int corner = 0; corner < (1 << nax); ++corner) {
         double ww = 1.0;
-        int ix = i0[0] + (corner & 1), iy = 0, iz;
-        ww *= (corner & 1) ? fr[0] : 1.0 - fr[0];
-        if (nax == 2) {
-            iz = i0[1] + ((corner >> 1) & 1);
-            ww *= ((corner >> 1) & 1) ? fr[1] : 1.0 - fr[1];
-        } else {
-            iy = i0[1] + ((corner >> 1) & 1);
-            ww *= ((corner >> 1) & 1) ? fr[1] : 1.0 - fr[1];
-            iz = i0[2] + ((corner >> 2) & 1);
-            ww *= ((corner >> 2) & 1) ? fr[2] : 1.0 - fr[2];
+        int at[3] = {0, 0, 0};
+        for (int a = 0; a < nax; ++a) {
+            const int up = (corner >> a) & 1;
+            at[a] = i0[a] + up;
+            ww *= up ? fr[a] : 1.0 - fr[a];
         }
         if (ww == 0.0) continue;
-        idx[k] = (int)(((long long)iz * d.Ny + iy) * d.P + ix);
-        w[k] = (float)ww;
+        tap[k].x = at[0];
+        tap[k].y = nax == 2 ? 0 : at[1];
+        tap[k].z = nax == 2 ? at[1] : at[2];
+        tap[k].w = (float)ww;
         ++k;
     }
     *n = k;
     return true;
 }
 
-wave_status_t build_taps(const Dims& d, const Tiling& t, int nshot, int npts, const float* xyz, HostTaps& out)
+wave_status_t build_taps(const Dims& d, const Tiling& t, int nshot, int npts, const float* xyz, bool count_only,
+                         HostTaps& out)
 {
     out = HostTaps();
     out.npts = npts;
     const long long cps = t.cells_per_shot();
     const long long npts_all = (long long)nshot * npts;
-    std::vector<int> cell_of;
-    std::vector<int> idx_pt, ab_pt;
-    std::vector<float> w_pt;
+    out.npt_start = (size_t)npts_all + 1;
+    PointTap tap[8];
+    int n = 0;
+    if (count_only) {
+        for (long long pt = 0; pt < npts_all; ++pt) {
+            if (!point_taps(d, xyz + pt * d.ndim, tap, &n)) return WAVE_ERR_GEOMETRY;
+            out.ntap += n;
+        }
+        return WAVE_OK;
+    }
+    // the taps in point order, and how many each cell holds
+    struct Item {
+        int cell, idx, ab;
+        float w;
+    };
+    std::vector<Item> item;
+    item.reserve(npts_all * (d.ndim == 3 ? 2 : 4));
     out.pt_start.resize(npts_all + 1);
-    cell_of.reserve(npts_all * 2);
-    int tmp_idx[8];
-    float tmp_w[8];
+    out.cell_start.assign(nshot * cps + 1, 0);
     for (int s = 0; s < nshot; ++s) {
         for (int p = 0; p < npts; ++p) {
             const long long pt = (long long)s * npts + p;
-            out.pt_start[pt] = (int)idx_pt.size();
-            int n = 0;
-            if (!point_taps(d, xyz + pt * d.ndim, tmp_idx, tmp_w, &n)) return WAVE_ERR_GEOMETRY;
+            out.pt_start[pt] = (int)item.size();
+            if (!point_taps(d, xyz + pt * d.ndim, tap, &n)) return WAVE_ERR_GEOMETRY;
             for (int k = 0; k < n; ++k) {
-                const int i = tmp_idx[k];
-                const int x = i % d.P;
-                const int r = i / d.P;
-                const int y = r % d.Ny;
-                const int z = r / d.Ny;
                 // cells in (shot, cx, cy, cz) order with cz fastest
-                const long long cell = (((long long)s * t.ncx + x / t.TX) * t.ncy + y / t.TY) * t.ncz + z / t.TZc;
-                cell_of.push_back((int)cell);
-                idx_pt.push_back(i);
-                w_pt.push_back(tmp_w[k]);
-                ab_pt.push_back((int)((long long)s * d.nt * npts + p));
+                const long long cell =
+                    (((long long)s * t.ncx + tap[k].x / t.TX) * t.ncy + tap[k].y / t.TY) * t.ncz + tap[k].z / t.TZc;
+                item.push_back({(int)cell, (int)(((long long)tap[k].z * d.Ny + tap[k].y) * d.P + tap[k].x),
+                                (int)((long long)s * d.nt * npts + p), tap[k].w});
+                ++out.cell_start[cell + 1];
             }
         }
     }
-    out.pt_start[npts_all] = (int)idx_pt.size();
-    const size_t ntap = idx_pt.size();
+    out.pt_start[npts_all] = (int)item.size();
+    const size_t ntap = out.ntap = item.size();
     // Stable counting sort of the taps by cell.
-    out.cell_start.assign(nshot * cps + 1, 0);
-    for (size_t j = 0; j < ntap; ++j) out.cell_start[cell_of[j] + 1]++;
     for (long long i = 0; i < nshot * cps; ++i) out.cell_start[i + 1] += out.cell_start[i];
-    std::vector<int> fill(out.cell_start.begin(), out.cell_start.end() - 1);
+    std::vector<int> fill(out.cell_start.begin(), out.cell_start.end() - 1), order(ntap);
+    for (size_t j = 0; j < ntap; ++j) order[fill[item[j].cell]++] = (int)j;
+    // Inside a cell, taps of the same grid point become adjacent (stable by
+    // point order), so one thread can own each injected point.
+    const auto before = [&](int x, int y) { return item[x].idx < item[y].idx; };
+    for (size_t b = 0; b < ntap;) {
+        const size_t e = out.cell_start[item[order[b]].cell + 1];
+        if (!std::is_sorted(order.begin() + b, order.begin() + e, before))
+            std::stable_sort(order.begin() + b, order.begin() + e, before);
+        b = e;
+    }
     out.idx.resize(ntap);
     out.w.resize(ntap);
     out.ab.resize(ntap);
     out.slot.resize(ntap);
-    std::vector<int> order(ntap);
-    for (size_t j = 0; j < ntap; ++j) order[fill[cell_of[j]]++] = (int)j;
-    // Inside a cell, taps of the same grid point become adjacent (stable by
-    // point order), so one thread can own each injected point.
-    for (long long c = 0; c < nshot * cps; ++c)
-        std::stable_sort(order.begin() + out.cell_start[c], order.begin() + out.cell_start[c + 1],
-                         [&](int x, int y) { return idx_pt[x] < idx_pt[y]; });
     for (size_t pos = 0; pos < ntap; ++pos) {
-        const int j = order[pos];
-        out.idx[pos] = idx_pt[j];
-        out.w[pos] = w_pt[j];
-        out.ab[pos] = ab_pt[j];
-        out.slot[pos] = j;
+        const Item& it = item[order[pos]];
+        out.idx[pos] = it.idx;
+        out.w[pos] = it.w;
+        out.ab[pos] = it.ab;
+        out.slot[pos] = order[pos];
     }
     return WAVE_OK;
 }
