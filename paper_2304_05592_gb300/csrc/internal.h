@@ -104,6 +104,7 @@ struct StepArgs {
     int ncx, ncy, ncz;   // tap cells per shot
     int TZc;             // tap cell height
     // injection into unew (forward: sources with q^n; adjoint: receivers with r^k)
+    int planes;          // 3D plane ring: planes per CTA (set by its launcher)
     TapList inj;
     const float* amp_a;  // amplitude array [nshot][nt][npts]
     const float* amp_b;  // subtracted from amp_a (NULL = none)

@@ -1288,7 +1288,7 @@ __global__ void __launch_bounds__(32 * TY) k_step3d(const StepArgs a)
 
 // ---------------------------------------------------------------------------
 // 3D step fed by TMA.  Tile = 128 (x) by TY (y) points, CTA = 32 x TY threads
-// (4 x points per thread) marching over TZC planes in z.  Every xy plane of u
+// (4 x points per thread) marching over a.planes planes in z.  Every xy plane of u
 // with its 4-point halo ((TY+8) x 136 floats) arrives by one 5D bulk tensor
 // load into a ring of NR shared-memory slots: planes z..z+4 are resident
 // while planes up to z+NR-1 are in flight.  Each thread keeps the 9 planes
@@ -1298,7 +1298,7 @@ __global__ void __launch_bounds__(32 * TY) k_step3d(const StepArgs a)
 // as centre: one barrier per plane.  Sponge depths in x and y are fixed per
 // thread.  Waits are bounded; on a timeout the CTA records kErrTimeout, lets
 // its issued copies land and returns.
-template <int TY, int TZC, int NR, bool ADJ, int PF = 0>
+template <int TY, int NR, bool ADJ, int PF = 0>
 __global__ void __launch_bounds__(32 * TY, TY <= 8 ? 2 : 1) k_step3d_tma(const __grid_constant__ StepMaps mp,
                                                                         const StepArgs a)
 {
@@ -1308,6 +1308,7 @@ __global__ void __launch_bounds__(32 * TY, TY <= 8 ? 2 : 1) k_step3d_tma(const _
     __shared__ __align__(8) uint64_t bar[NR];
     float* ring = reinterpret_cast<float*>(dyn + ((128u - (smem_u32(dyn) & 127u)) & 127u));
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 32 + tx;
+    const int TZC = a.planes;
     const int x0 = blockIdx.x * kTX, y0 = blockIdx.y * TY;
     const int ntz = (a.Nz + TZC - 1) / TZC;
     const int shot = blockIdx.z / ntz, tzi = blockIdx.z - shot * ntz;
@@ -1763,7 +1764,7 @@ static const Variant2D k3D[] = {{0, 32, 8, 0, 0},  {6, 32, 8, 7, 0},  {6, 64, 8,
                                 {6, 64, 16, 7, 0}, {6, 64, 8, 10, 0}, {6, 32, 8, 10, 0}, {6, 96, 8, 10, 0},
                                 {6, 64, 8, 10, 1}, {6, 64, 8, 12, 1}, {6, 96, 8, 12, 1}, {6, 64, 8, 8, 4},
                                 {6, 64, 8, 7, 5},  {6, 96, 8, 8, 4},  {6, 76, 8, 10, 0},
-                                {6, 76, 8, 12, 0}, {6, 76, 8, 8, 0}};
+                                {6, 76, 8, 12, 0}, {6, 0, 8, 8, 0}};
 static int g_selected[3] = {-1, -1, -1};
 static const int kDefaultVariant[3] = {44, 42, 16};
 
@@ -1817,22 +1818,45 @@ static void launch_3d_ws(bool adjoint, const StepArgs& a, const StepMaps* maps, 
     else k_step3d_ws<TY, TZC, NR, false><<<grid, dim3(32, TY), smem, s>>>(*maps, a);
 }
 
-template <int TY, int TZC, int NR, int PF = 0>
-static void launch_3d_tma(bool adjoint, const StepArgs& a, const StepMaps* maps, cudaStream_t s)
+// Planes per CTA of the plane-ring kernel: a CTA costs its planes and about 6
+// more (the ring's first 8 planes, the tail), and the launch as many rounds of
+// those as its CTAs fill (2 per SM), so the chunk count with the fewest rounds x
+// planes is taken.  Chunks are multiples of the tap cells' 4 planes.  480 x 480 x
+// 380: 5 chunks of 76 planes (3.95 rounds), 293 us per step; 2 shots of 141 x 123 x
+// 107: 4 chunks of 28 planes instead of 2 of 76, which left half the SMs idle.
+static int planes_per_cta(const StepArgs& a, int TY)
+{
+    const long long columns = (long long)a.ncx * ((a.Ny + TY - 1) / TY) * a.nshot, slots = 2LL * num_sms();
+    int best = a.Nz;
+    long long least = 0;
+    for (int nc = 1; nc <= (a.Nz + 7) / 8; ++nc) {
+        const int tzc = ((a.Nz + nc - 1) / nc + 3) / 4 * 4, chunks = (a.Nz + tzc - 1) / tzc;
+        const long long cost = (columns * chunks + slots - 1) / slots * (std::min(tzc, a.Nz) + 6);
+        if (nc == 1 || cost < least) {
+            least = cost;
+            best = tzc;
+        }
+    }
+    return best;
+}
+
+// planes = 0: planes_per_cta's choice
+template <int TY, int NR, int PF = 0>
+static void launch_3d_tma(int planes, bool adjoint, const StepArgs& args, const StepMaps* maps, cudaStream_t s)
 {
     constexpr size_t smem = (size_t)NR * (TY + 8) * (kTX + 8) * 4 + (size_t)(PF > 0 ? (PF + 1) * 2 * 32 * TY * 16 : 0) +
                             128;
     static bool configured[kMaxDev] = {};
     if (first_on_device(configured)) {
-        cudaFuncSetAttribute(k_step3d_tma<TY, TZC, NR, false, PF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-        cudaFuncSetAttribute(k_step3d_tma<TY, TZC, NR, true, PF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
+        cudaFuncSetAttribute(k_step3d_tma<TY, NR, false, PF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(k_step3d_tma<TY, NR, true, PF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     }
-    const int ntz = (a.Nz + TZC - 1) / TZC;
+    StepArgs a = args;
+    a.planes = planes > 0 ? planes : planes_per_cta(a, TY);
+    const int ntz = (a.Nz + a.planes - 1) / a.planes;
     dim3 grid(a.ncx, (a.Ny + TY - 1) / TY, ntz * a.nshot);
-    if (adjoint) k_step3d_tma<TY, TZC, NR, true, PF><<<grid, dim3(32, TY), smem, s>>>(*maps, a);
-    else k_step3d_tma<TY, TZC, NR, false, PF><<<grid, dim3(32, TY), smem, s>>>(*maps, a);
+    if (adjoint) k_step3d_tma<TY, NR, true, PF><<<grid, dim3(32, TY), smem, s>>>(*maps, a);
+    else k_step3d_tma<TY, NR, false, PF><<<grid, dim3(32, TY), smem, s>>>(*maps, a);
 }
 
 template <int TZ, int BZ, int G, bool ADJ>
@@ -2042,22 +2066,22 @@ static void launch_step_raw(const Tiling& t, int ndim, bool adjoint, const StepA
         }
     } else {
         switch (a.dmv ? 0 : t.v3) {  // the Born source is carried by the z-march kernel only
-        case 1: launch_3d_tma<8, 32, 7>(adjoint, a, maps, s); break;
-        case 2: launch_3d_tma<8, 64, 7>(adjoint, a, maps, s); break;
-        case 3: launch_3d_tma<16, 32, 7>(adjoint, a, maps, s); break;
-        case 4: launch_3d_tma<16, 64, 7>(adjoint, a, maps, s); break;
-        case 5: launch_3d_tma<8, 64, 10>(adjoint, a, maps, s); break;
-        case 6: launch_3d_tma<8, 32, 10>(adjoint, a, maps, s); break;
-        case 7: launch_3d_tma<8, 96, 10>(adjoint, a, maps, s); break;
+        case 1: launch_3d_tma<8, 7>(32, adjoint, a, maps, s); break;
+        case 2: launch_3d_tma<8, 7>(64, adjoint, a, maps, s); break;
+        case 3: launch_3d_tma<16, 7>(32, adjoint, a, maps, s); break;
+        case 4: launch_3d_tma<16, 7>(64, adjoint, a, maps, s); break;
+        case 5: launch_3d_tma<8, 10>(64, adjoint, a, maps, s); break;
+        case 6: launch_3d_tma<8, 10>(32, adjoint, a, maps, s); break;
+        case 7: launch_3d_tma<8, 10>(96, adjoint, a, maps, s); break;
         case 8: launch_3d_ws<8, 64, 10>(adjoint, a, maps, s); break;
         case 9: launch_3d_ws<8, 64, 12>(adjoint, a, maps, s); break;
         case 10: launch_3d_ws<8, 96, 12>(adjoint, a, maps, s); break;
-        case 11: launch_3d_tma<8, 64, 8, 3>(adjoint, a, maps, s); break;
-        case 12: launch_3d_tma<8, 64, 7, 4>(adjoint, a, maps, s); break;
-        case 13: launch_3d_tma<8, 96, 8, 3>(adjoint, a, maps, s); break;
-        case 14: launch_3d_tma<8, 76, 10>(adjoint, a, maps, s); break;
-        case 15: launch_3d_tma<8, 76, 12>(adjoint, a, maps, s); break;
-        case 16: launch_3d_tma<8, 76, 8>(adjoint, a, maps, s); break;
+        case 11: launch_3d_tma<8, 8, 3>(64, adjoint, a, maps, s); break;
+        case 12: launch_3d_tma<8, 7, 4>(64, adjoint, a, maps, s); break;
+        case 13: launch_3d_tma<8, 8, 3>(96, adjoint, a, maps, s); break;
+        case 14: launch_3d_tma<8, 10>(76, adjoint, a, maps, s); break;
+        case 15: launch_3d_tma<8, 12>(76, adjoint, a, maps, s); break;
+        case 16: launch_3d_tma<8, 8>(0, adjoint, a, maps, s); break;
         default: {
             const int ntz = (a.Nz + 31) / 32;
             dim3 grid(t.ncx, t.ncy, ntz * a.nshot);
