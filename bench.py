@@ -43,9 +43,9 @@ VARIANT_KERNEL = {(0, 18): ("k_step2d_sgt", "k_step2d_sgt<16,8,2,0,fwd>"),
                   (1, 16): ("k_step2d_sgt", "k_step2d_sgt<16,8,2,0,adj>"),
                   (1, 25): ("k_step2d_sgt", "k_step2d_sgt<16,8,2,1,adj>")}
 # shot-group TMA kernels with deeper rings and the adjoint's forward level by TMA
-for _k, _fl, _g in ((39, 9, 2), (40, 9, 4), (41, 17, 4), (42, 9, 8), (43, 17, 8), (44, 41, 4), (45, 33, 2), (46, 41, 8), (47, 49, 4)):
+for _k, _fl, _g in ((39, 9, 2), (40, 9, 4), (41, 17, 4), (42, 9, 8), (43, 17, 8), (44, 41, 4), (45, 33, 2), (46, 41, 8), (47, 49, 4), (48, 41, 2), (49, 41, 1)):
     VARIANT_KERNEL[(0, _k)] = ("k_step2d_sgt", "k_step2d_sgt<16,8,%d,%d,fwd>" % (_g, _fl))
-for _k, _fl, _g in ((37, 5, 2), (38, 13, 2), (39, 13, 4), (40, 5, 4), (41, 69, 4), (42, 101, 4), (43, 37, 4), (44, 101, 8), (45, 45, 4), (46, 101, 2)):
+for _k, _fl, _g in ((37, 5, 2), (38, 13, 2), (39, 13, 4), (40, 5, 4), (41, 69, 4), (42, 101, 4), (43, 37, 4), (44, 101, 8), (45, 45, 4), (46, 101, 2), (47, 101, 1)):
     VARIANT_KERNEL[(1, _k)] = ("k_step2d_sgt", "k_step2d_sgt<16,8,%d,%d,adj>" % (_g, _fl))
 # the z-window kernels (step2d_zw.cu): (TZ, BZ, G) of forward variants 33-38 and adjoint variants 31-36
 for _i, _c in enumerate([(16, 4, 2), (16, 4, 4), (16, 2, 2), (32, 8, 2), (32, 4, 2), (16, 8, 2)]):

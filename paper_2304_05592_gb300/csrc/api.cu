@@ -436,15 +436,13 @@ float sponge_coefficient(const Dims& d)
 }
 
 // Time of one step of all shots with a launch per step (us), to weigh against
-// the on-chip loop's estimate.  Measured with the default kernels: 4.15 / 4.7 us
-// for one shot (no faster than launches queue), 1.95 / 2.85 us more for each of
-// the up to 4 shots a CTA works through (9.6 / 13.6 us at 4 shots of 480 x 280,
-// 11.0 / 14.1 us at 16 of 336 x 208), then the tile kernels' rate (16.6 / 20 us
-// at 32 shots of 592 x 336).
+// the on-chip loop's estimate: the tile kernels' time, but no less than launches
+// take to queue (4.15 / 4.7 us).
 float launched_step_us(const Dims& d, int nshot, bool adjoint)
 {
-    const float pts = (float)d.Nz * d.Nx * nshot, g = (float)std::min(nshot, 4);
-    return adjoint ? std::max({4.7f, 2.2f + 2.85f * g, 3.1e-6f * pts}) : std::max({4.15f, 2.0f + 1.95f * g, 2.55e-6f * pts});
+    float tiles = 0.0f;
+    shot_group(d, nshot, adjoint, &tiles);
+    return std::max(tiles, adjoint ? 4.7f : 4.15f);
 }
 
 // Decides between the on-chip time loop and the per-step kernels, per
@@ -458,10 +456,10 @@ void choose_chip(Layout& L)
         ChipPlan p;
         if (asked || !set) p = chip_plan(L.d, L.t, L.nshot, mode, inj, gat);
         // (the estimates are good to 10 %; where they nearly meet the launches have the better of it)
-        if (p.C && !asked && 1.15f * p.step_us >= launched_step_us(L.d, L.nshot, which == 1)) p.C = 0;
+        if (p.C && !asked && 1.1f * p.step_us >= launched_step_us(L.d, L.nshot, which == 1)) p.C = 0;
         if (L.nbuf >= 32768) p.C = 0;  // buffer indices travel as 16-bit numbers
         if (p.C) v = chip_variant(which);
-        else if (asked) v = default_variant(which);
+        else if (asked) v = group_variant(which == 1, shot_group(L.d, L.nshot, which == 1, nullptr));
         return p;
     };
     const HostTaps none;

@@ -182,6 +182,10 @@ int chip_variant(int which);              // the kind-8 entry of the 2D tables
 
 // Remembers the last failing CUDA call of this thread (profile.cu).
 void note_cuda_error(cudaError_t e);
+int group_variant(bool adjoint, int g);   // the default 2D kernel with g = 1, 2 or 4 shots per CTA
+// Shots per CTA for the shot-group kernels on this grid (1, 2 or 4) and the
+// estimated time of a step (us).
+int shot_group(const Dims& d, int nshot, bool adjoint, float* step_us);
 
 // Launch accounting and sampled per-launch timing of the stencil kernels
 // (profile.cu).  Every launcher above calls count_launch(); launch_step wraps

@@ -1743,7 +1743,8 @@ static const Variant2D kFwd2D[] = {{0, 32, 4, 0, 0}, {1, 48, 6, 2, 0}, {1, 32, 4
                                    {4, 16, 8, 2, 4},  {7, 16, 4, 0, 2}, {7, 16, 4, 1, 4}, {7, 16, 2, 2, 2},
                                    {7, 32, 8, 3, 2},  {7, 32, 4, 4, 2}, {7, 16, 8, 5, 2}, {4, 16, 8, 9, 2},
                                    {4, 16, 8, 9, 4},  {4, 16, 8, 17, 4}, {4, 16, 8, 9, 8}, {4, 16, 8, 17, 8}, {4, 16, 8, 41, 4},
-                                   {4, 16, 8, 33, 2},  {4, 16, 8, 41, 8}, {4, 16, 8, 49, 4}, {8, 16, 8, 0, 0}};
+                                   {4, 16, 8, 33, 2},  {4, 16, 8, 41, 8}, {4, 16, 8, 49, 4}, {4, 16, 8, 41, 2}, {4, 16, 8, 41, 1},
+                                   {8, 16, 8, 0, 0}};
 static const Variant2D kAdj2D[] = {{0, 32, 4, 0, 0}, {1, 24, 3, 3, 0}, {1, 16, 2, 4, 0}, {1, 32, 4, 2, 0},
                                    {2, 32, 8, 0, 4}, {2, 16, 8, 0, 4}, {2, 32, 8, 0, 8}, {2, 16, 8, 0, 2},
                                    {3, 24, 4, 1, 0}, {3, 24, 4, 2, 0}, {3, 48, 4, 2, 0}, {3, 16, 8, 2, 0},
@@ -1755,8 +1756,9 @@ static const Variant2D kAdj2D[] = {{0, 32, 4, 0, 0}, {1, 24, 3, 3, 0}, {1, 16, 2
                                    {7, 16, 4, 1, 4}, {7, 16, 2, 2, 2}, {7, 32, 8, 3, 2},  {7, 32, 4, 4, 2},
                                    {7, 16, 8, 5, 2}, {4, 16, 8, 5, 2}, {4, 16, 8, 13, 2}, {4, 16, 8, 13, 4},
                                    {4, 16, 8, 5, 4}, {4, 16, 8, 69, 4}, {4, 16, 8, 101, 4}, {4, 16, 8, 37, 4},
-                                   {4, 16, 8, 101, 8}, {4, 16, 8, 45, 4}, {4, 16, 8, 101, 2}, {8, 16, 8, 0, 0}};
-// 3D variants (which = 2; TZ = planes per CTA, R = tile rows in y, NST = ring
+                                   {4, 16, 8, 101, 8}, {4, 16, 8, 45, 4}, {4, 16, 8, 101, 2}, {4, 16, 8, 101, 1},
+                                   {8, 16, 8, 0, 0}};
+// 3D variants (which = 2; TZ = planes per CTA (0: chosen per grid), R = tile rows in y, NST = ring
 // slots, G = 1 for the ring without block barriers, G = PF + 1 for the ring
 // whose model and previous level arrive PF planes ahead by cp.async): kind 0
 // is the z-march with a shared-memory halo plane, kind 6 the TMA plane ring.
@@ -1791,6 +1793,11 @@ int current_variant(int which)
 }
 
 int default_variant(int which) { return kDefaultVariant[which]; }
+
+int group_variant(bool adjoint, int g)
+{
+    return adjoint ? (g == 1 ? 47 : (g == 2 ? 46 : 42)) : (g == 1 ? 49 : (g == 2 ? 48 : 44));
+}
 
 int chip_variant(int which) { return variant_count(which) - 1; }
 
@@ -2017,6 +2024,8 @@ static void launch_step_raw(const Tiling& t, int ndim, bool adjoint, const StepA
             case 45: launch_2d_group_tma<16, 8, 2, false, 1 | 32>(a, maps, s); break;
             case 46: launch_2d_group_tma<16, 8, 8, false, 9 | 32>(a, maps, s); break;
             case 47: launch_2d_group_tma<16, 8, 4, false, 17 | 32>(a, maps, s); break;
+            case 48: launch_2d_group_tma<16, 8, 2, false, 9 | 32>(a, maps, s); break;
+            case 49: launch_2d_group_tma<16, 8, 1, false, 9 | 32>(a, maps, s); break;
             default: launch_2d_direct<32, 8, false>(a, s); break;
             }
         } else {
@@ -2061,6 +2070,7 @@ static void launch_step_raw(const Tiling& t, int ndim, bool adjoint, const StepA
             case 44: launch_2d_group_tma<16, 8, 8, true, 5 | 32 | 64>(a, maps, s); break;
             case 45: launch_2d_group_tma<16, 8, 4, true, 13 | 32>(a, maps, s); break;
             case 46: launch_2d_group_tma<16, 8, 2, true, 5 | 32 | 64>(a, maps, s); break;
+            case 47: launch_2d_group_tma<16, 8, 1, true, 5 | 32 | 64>(a, maps, s); break;
             default: launch_2d_direct<32, 8, true>(a, s); break;
             }
         }

@@ -44,6 +44,39 @@ void remember_tuning(const Dims& d, int nshot, int vf, int va)
     g_tuned[std::make_tuple(d.Nx, d.Nz, nshot)] = std::make_pair(vf, va);
 }
 
+// A CTA sets its tile up once and then takes its group's shots one after the
+// other; 3 CTAs fit an SM.  Larger groups spread the set-up over more shots,
+// smaller ones fill the GPU and shorten the chain: with groups of 4 throughout, 8
+// shots of 592 x 336 (210 CTAs on 456 slots) ran at 10.7 / 14.6 us per step, with
+// singly (840 CTAs) at 6.4 / 7.8 us.  Model of a step (us) with N CTAs: the chain
+// of one CTA, a little longer with neighbours on the SM, or the GPU's rate over
+// all of them, whichever is longer; 36 timings (592 x 336 with 1 to 32 shots, 1280 x
+// 580 with 1 and 4, groups of 1, 2 and 4) lie within 10 % but for 24.5 and 32.6 us
+// (predicted 21.7 and 27.5) at 32 shots singly.
+int shot_group(const Dims& d, int nshot, bool adjoint, float* step_us)
+{
+    static const float kChain[2][3][2] = {{{4.6f, 0.0f}, {6.2f, 0.0021f}, {9.4f, 0.006f}},
+                                          {{5.6f, 0.0019f}, {8.0f, 0.0035f}, {13.3f, 0.005f}}};
+    static const float kRate[2][3][2] = {{{0.9f, 0.0062f}, {1.0f, 0.0104f}, {3.5f, 0.0172f}},
+                                         {{1.3f, 0.0078f}, {1.5f, 0.0122f}, {5.5f, 0.0172f}}};
+    const float tiles = (float)((d.Nx + kTX - 1) / kTX) * ((d.Nz + 15) / 16);
+    int best = 4;
+    float least = 0.0f;
+    for (int k = 2; k >= 0; --k) {
+        const int g = 1 << k;
+        const float n = tiles * ((nshot + g - 1) / g), *c = kChain[adjoint][k], *r = kRate[adjoint][k];
+        // (a group larger than the batch is as long as the batch)
+        const float chain = nshot < g ? kChain[adjoint][0][0] + (c[0] - kChain[adjoint][0][0]) * (nshot - 1) / (g - 1) : c[0];
+        const float t = std::max(chain + c[1] * n, nshot < g ? 0.0f : r[0] + r[1] * n);
+        if (k == 2 || t < least) {
+            best = g;
+            least = t;
+        }
+    }
+    if (step_us) *step_us = least;
+    return best;
+}
+
 Tiling choose_tiling(const Dims& d, int nshot)
 {
     Tiling t;
@@ -63,6 +96,10 @@ Tiling choose_tiling(const Dims& d, int nshot)
             if (!variant_forced(0)) t.vf = it->second.first;
             if (!variant_forced(1)) t.va = it->second.second;
             t.set_f = t.set_a = true;
+        }
+        if (nshot > 0) {
+            if (!t.set_f) t.vf = group_variant(false, shot_group(d, nshot, false, nullptr));
+            if (!t.set_a) t.va = group_variant(true, shot_group(d, nshot, true, nullptr));
         }
     } else {
         t.TY = 8;
