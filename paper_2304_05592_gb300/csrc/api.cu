@@ -1068,16 +1068,41 @@ wave_status_t wave_born(const wave_grid_t* grid, const float* vel, int nshot, in
     if (nshot == 0) return clear_header(L, work, work_bytes, s);
     if (!vel || !dm || (nsrc && !wavelet) || (nrec && !data)) return WAVE_ERR_ARG;
     if ((st = check_work(L, work, work_bytes))) return st;
-    L.t.vf = 0;  // the direct 2D kernel carries the scattering source
+    const int group = shot_group(L.d, nshot, true, nullptr);  // (a Born step weighs like an adjoint one)
+    L.t.vf = default_variant(0);  // 16-row boxes in the maps, as the Born kernel's tiles
     if ((st = setup(L, vel, s))) return st;
     launch_prep_dm(L.d, dm, L.kap, L.dmv, s);
     const size_t fb = L.field() * sizeof(float);
     CK(cudaMemsetAsync(L.buf(0), 0, 5 * fb, s));
     const size_t nrow = L.hr.idx.size();
     if (nrow) CK(cudaMemsetAsync(L.slots_rec, 0, nrow * sizeof(float), s));
-    int cur = 0, prev = 1, nxt = 2;  // background u^n, u^{n-1}, free
     int dcur = L.iA0, dprev = L.iA0 + 1;
-    for (int n = 0; n + 1 < L.d.nt; ++n) {
+    if (L.d.ndim == 2) {
+        int cur = 0, prev = 1;  // background u^n; u^{n-1}, overwritten by u^{n+1}
+        for (int n = 0; n + 1 < L.d.nt; ++n) {
+            StepArgs a = base_args(L);
+            a.u_buf = cur;
+            a.prev_buf = prev;
+            a.unew = L.buf(prev);
+            a.dmv = L.dmv;
+            a.group = group;
+            if (nsrc > 0 && L.ts.l.ntap > 0) {
+                a.inj = L.ts.l;
+                a.amp_a = wavelet;
+                a.amp_row = n;
+            }
+            if (nrec > 0 && L.tr.l.ntap > 0) {
+                a.gat = L.tr.l;
+                a.slots = L.slots_rec;
+                a.slot_row = n + 1;
+            }
+            launch_born2d(a, dcur, dprev, L.buf(dprev), &L.maps, s);
+            std::swap(cur, prev);
+            std::swap(dcur, dprev);
+        }
+    }
+    int cur = 0, prev = 1, nxt = 2;  // 3D: background u^n, u^{n-1}, free
+    for (int n = 0; n + 1 < L.d.nt && L.d.ndim == 3; ++n) {
         fwd_step(L, cur, prev, nxt, n, wavelet, false, nullptr, nullptr, s);  // u^{n+1}
         StepArgs a = base_args(L);
         a.u = L.buf(dcur);

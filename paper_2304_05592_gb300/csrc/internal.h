@@ -100,11 +100,12 @@ struct StepArgs {
     long long cell;
     int nb, nx, ny, nz;
     int nshot;
+    int group;           // Born step: shots per CTA (1 to 4)
     float ceps;          // eps = kap * ceps * depth^2 is eta dt v^2 / 2
     int ncx, ncy, ncz;   // tap cells per shot
     int TZc;             // tap cell height
-    // injection into unew (forward: sources with q^n; adjoint: receivers with r^k)
     int planes;          // 3D plane ring: planes per CTA (set by its launcher)
+    // injection into unew (forward: sources with q^n; adjoint: receivers with r^k)
     TapList inj;
     const float* amp_a;  // amplitude array [nshot][nt][npts]
     const float* amp_b;  // subtracted from amp_a (NULL = none)
@@ -169,6 +170,9 @@ struct Variant2D {
 // consecutive rows in registers (G shots per CTA; NST = configuration index
 // of launch_step2d_zw, step2d_zw.cu).
 void launch_step2d_zw(int config, bool adjoint, const StepArgs& a, const StepMaps* maps, cudaStream_t s);
+// 2D Born step (born2d.cu): u^{n+1} over u^{n-1} (a.unew) and the scattered level
+// over pnew, gathering the latter; boxes of 16-row tiles in the forward maps.
+void launch_born2d(const StepArgs& a, int p_buf, int pprev_buf, float* pnew, const StepMaps* maps, cudaStream_t s);
 // Number of per-shot/per-group gradient accumulators the adjoint step fills.
 int gradient_accumulators(const struct Tiling& t, int ndim, int nshot);
 int persistent_slots(int v, int ncx, int ntz, int nshot);  // adjoint variant v of kind 5
@@ -178,14 +182,14 @@ int current_variant(int which);           // the selected or default variant
 int select_variant(int which, int v);     // v = -1 restores the default; 0 on success
 bool variant_forced(int which);           // true after wave_set_variant(which, v >= 0)
 int default_variant(int which);
-int chip_variant(int which);              // the kind-8 entry of the 2D tables
-
-// Remembers the last failing CUDA call of this thread (profile.cu).
-void note_cuda_error(cudaError_t e);
 int group_variant(bool adjoint, int g);   // the default 2D kernel with g = 1, 2 or 4 shots per CTA
 // Shots per CTA for the shot-group kernels on this grid (1, 2 or 4) and the
 // estimated time of a step (us).
 int shot_group(const Dims& d, int nshot, bool adjoint, float* step_us);
+int chip_variant(int which);              // the kind-8 entry of the 2D tables
+
+// Remembers the last failing CUDA call of this thread (profile.cu).
+void note_cuda_error(cudaError_t e);
 
 // Launch accounting and sampled per-launch timing of the stencil kernels
 // (profile.cu).  Every launcher above calls count_launch(); launch_step wraps
