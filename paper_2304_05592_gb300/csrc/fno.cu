@@ -68,10 +68,9 @@ __global__ void k_tables(int Nz, int Nx, int mz, int mx, float* tf, float* ti, f
 }
 
 // --- along x: out[r][n] = sum_x in[r][x] tab[x][n], n < 2 mx ------------------
-// CTA = 256 threads, kDxRows rows; thread (tr, tn) owns rows kDxRq tr ..
-// kDxRq tr + kDxRq - 1 and outputs 4 tn .. 4 tn + 3, accumulated over x in
-// chunks of 32 staged in shared memory (rows padded to 33 floats: conflict-free
-// in both directions).  The chunks are double-buffered: chunk c + 1 is loaded
+// CTA = 256 threads, kDxRows rows; thread (tr, tn) owns rows tr, tr + 32, ...
+// and outputs 4 tn .. 4 tn + 3 (in pairs, FFMA2), accumulated over x in chunks of
+// 32 staged in shared memory (rows padded to 36 floats) and read four x at a time.  The chunks are double-buffered: chunk c + 1 is loaded
 // into registers while chunk c is summed, then stored to the other buffer, one
 // block barrier per chunk.  128 rows per CTA put a 65536-row transform on the
 // GPU in one wave.
@@ -82,15 +81,15 @@ template <typename T>
 __global__ void __launch_bounds__(256, 4) k_dft_x(long long rows, int Nx, int n2, const T* __restrict__ in,
                                                const float* __restrict__ tab, float* __restrict__ out)
 {
-    __shared__ float sv[2][kDxRows][kDxChunk + 1];
+    __shared__ __align__(16) float sv[2][kDxRows][kDxChunk + 4];
     __shared__ __align__(16) float st[2][kDxChunk][32];
     const int tid = threadIdx.x, tn = tid & 7, tr = tid >> 3;
     const long long r0 = (long long)blockIdx.x * kDxRows;
-    float acc[kDxRq][4];
+    float2 acc[kDxRq][2];  // outputs in pairs
 #pragma unroll
     for (int q = 0; q < kDxRq; ++q)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[q][c] = 0.0f;
+        for (int c = 0; c < 2; ++c) acc[q][c] = make_float2(0.0f, 0.0f);
     float pv[kDxPv], pt[kDxPt];
     auto load = [&](int xc) {
 #pragma unroll
@@ -124,16 +123,23 @@ __global__ void __launch_bounds__(256, 4) k_dft_x(long long rows, int Nx, int n2
     for (int xc = 0; xc < Nx; xc += kDxChunk, q ^= 1) {
         const bool more = xc + kDxChunk < Nx;
         if (more) load(xc + kDxChunk);  // in flight during the sums below
-#pragma unroll 4
-        for (int x = 0; x < kDxChunk; ++x) {
-            const float4 t = *reinterpret_cast<const float4*>(&st[q][x][4 * tn]);
+#pragma unroll 2
+        for (int x = 0; x < kDxChunk; x += 4) {
+            float v[kDxRq][4];
 #pragma unroll
             for (int r = 0; r < kDxRq; ++r) {
-                const float a = sv[q][kDxRq * tr + r][x];
-                acc[r][0] = fmaf(a, t.x, acc[r][0]);
-                acc[r][1] = fmaf(a, t.y, acc[r][1]);
-                acc[r][2] = fmaf(a, t.z, acc[r][2]);
-                acc[r][3] = fmaf(a, t.w, acc[r][3]);
+                const float4 f = *reinterpret_cast<const float4*>(&sv[q][tr + 32 * r][x]);
+                v[r][0] = f.x, v[r][1] = f.y, v[r][2] = f.z, v[r][3] = f.w;
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float4 t = *reinterpret_cast<const float4*>(&st[q][x + j][4 * tn]);
+#pragma unroll
+                for (int r = 0; r < kDxRq; ++r) {
+                    const float2 w = make_float2(v[r][j], v[r][j]);
+                    acc[r][0] = __ffma2_rn(w, make_float2(t.x, t.y), acc[r][0]);
+                    acc[r][1] = __ffma2_rn(w, make_float2(t.z, t.w), acc[r][1]);
+                }
             }
         }
         if (more) store(q ^ 1);  // the buffer chunk c - 1 used: free since the last barrier
@@ -141,11 +147,96 @@ __global__ void __launch_bounds__(256, 4) k_dft_x(long long rows, int Nx, int n2
     }
 #pragma unroll
     for (int r = 0; r < kDxRq; ++r) {
-        const long long gr = r0 + kDxRq * tr + r;
+        const long long gr = r0 + tr + 32 * r;
         if (gr >= rows) continue;
+        const float o[4] = {acc[r][0].x, acc[r][0].y, acc[r][1].x, acc[r][1].y};
 #pragma unroll
         for (int c = 0; c < 4; ++c)
-            if (4 * tn + c < n2) out[(size_t)gr * n2 + 4 * tn + c] = acc[r][c];
+            if (4 * tn + c < n2) out[(size_t)gr * n2 + 4 * tn + c] = o[c];
+    }
+}
+
+// The same for FP32 rows of a multiple of 4 elements, 16-byte aligned, and 2 mx =
+// 32: a CTA of 128 threads takes 32 R rows, thread (tr, tn) rows tr + 32 r, r < R,
+// and outputs 8 tn .. 8 tn + 7.  Chunks of 16 x arrive by cp.async in two buffers;
+// per 4 x, R + 8 16-byte shared-memory loads feed 32 R products (16 R FFMA2), where
+// 4 x 4 blocks took 8 for 64 and were bound by them (l1tex 63 % busy, 88 us at
+// 65536 x 512).  The same order of x.
+constexpr int kDyChunk = 16, kDyS = kDyChunk + 4;
+template <int R>
+__global__ void __launch_bounds__(128, 4) k_dft_x8(long long rows, int Nx, const float* __restrict__ in,
+                                                   const float* __restrict__ tab, float* __restrict__ out)
+{
+    constexpr int kDyRows = 32 * R;
+    __shared__ __align__(16) float sv[2][kDyRows][kDyS];
+    __shared__ __align__(16) float st[2][kDyChunk][32];
+    const int tid = threadIdx.x, tn = tid & 3, tr = tid >> 2;
+    const long long r0 = (long long)blockIdx.x * kDyRows;
+    auto issue = [&](int xc, int q) {
+        const int p = 4 * (tid & 3);  // 4 pieces of 4 x per row and chunk
+        const int bytes = xc + p < Nx ? 16 : 0;
+#pragma unroll
+        for (int k = 0; k < kDyRows / 32; ++k) {
+            const int row = (tid >> 2) + 32 * k;
+            const float* src = in + (size_t)min(r0 + row, rows - 1) * Nx + (bytes ? xc + p : 0);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                             (uint32_t)__cvta_generic_to_shared(&sv[q][row][p])),
+                         "l"(src), "r"(bytes)
+                         : "memory");
+        }
+        const int x = tid >> 3, n = 4 * (tid & 7), tb = xc + x < Nx ? 16 : 0;  // 16 x 32 table entries, 4 each
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                         (uint32_t)__cvta_generic_to_shared(&st[q][x][n])),
+                     "l"(tab + (size_t)(tb ? xc + x : 0) * 32 + n), "r"(tb)
+                     : "memory");
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float2 acc[R][4];  // row r, outputs in pairs
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[r][c] = make_float2(0.0f, 0.0f);
+    issue(0, 0);
+    int q = 0;
+    for (int xc = 0; xc < Nx; xc += kDyChunk, q ^= 1) {
+        if (xc + kDyChunk < Nx) {
+            issue(xc + kDyChunk, q ^ 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int x = 0; x < kDyChunk; x += 4) {
+            float4 t[4][2];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                t[j][0] = *reinterpret_cast<const float4*>(&st[q][x + j][8 * tn]);
+                t[j][1] = *reinterpret_cast<const float4*>(&st[q][x + j][8 * tn + 4]);
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const float4 f = *reinterpret_cast<const float4*>(&sv[q][tr + 32 * r][x]);
+                const float v[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 w = make_float2(v[j], v[j]);
+                    acc[r][0] = __ffma2_rn(w, make_float2(t[j][0].x, t[j][0].y), acc[r][0]);
+                    acc[r][1] = __ffma2_rn(w, make_float2(t[j][0].z, t[j][0].w), acc[r][1]);
+                    acc[r][2] = __ffma2_rn(w, make_float2(t[j][1].x, t[j][1].y), acc[r][2]);
+                    acc[r][3] = __ffma2_rn(w, make_float2(t[j][1].z, t[j][1].w), acc[r][3]);
+                }
+            }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const long long gr = r0 + tr + 32 * r;
+        if (gr >= rows) continue;
+        float* o = out + (size_t)gr * 32 + 8 * tn;
+        *reinterpret_cast<float4*>(o) = make_float4(acc[r][0].x, acc[r][0].y, acc[r][1].x, acc[r][1].y);
+        *reinterpret_cast<float4*>(o + 4) = make_float4(acc[r][2].x, acc[r][2].y, acc[r][3].x, acc[r][3].y);
     }
 }
 
@@ -162,6 +253,14 @@ __device__ __forceinline__ float2 cfmac(float2 acc, float2 a, float2 b)
     return make_float2(fmaf(a.y, b.y, fmaf(a.x, b.x, acc.x)), fmaf(-a.x, b.y, fmaf(a.y, b.x, acc.y)));
 }
 
+// 8-byte asynchronous copy global -> shared; zeros if !ok.
+__device__ __forceinline__ void cp_async8(void* dst, const void* src, bool ok)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(ok ? 8 : 0)
+                 : "memory");
+}
+
 // out[b][a][kx] = sum_z in[b][z][kx] conj(E[z][a]); CTA per (b, 16 values of a).
 // Thread (h, q, kx) computes outputs (a0 + 4 q .. a0 + 4 q + 3, kx) over quarter h
 // of every 64-row chunk of z, so each in[z][kx] read from shared memory feeds
@@ -169,27 +268,39 @@ __device__ __forceinline__ float2 cfmac(float2 acc, float2 a, float2 b)
 __global__ void __launch_bounds__(256) k_dft_z(int Nz, int KZ, int mx, const float2* __restrict__ in,
                                                const float2* __restrict__ tz, float2* __restrict__ out)
 {
-    __shared__ float2 si[64][16];
-    __shared__ __align__(16) float2 se[64][16];
+    __shared__ __align__(16) float2 si[2][64][16], se[2][64][16];
     __shared__ float2 red[3][16][16];
     const int b = blockIdx.x, a0 = blockIdx.y * 16, tid = threadIdx.x;
     const int kx = tid & 15, q = (tid >> 4) & 3, h = tid >> 6;
+    // rows z0 .. z0 + 63 of the input and the table into buffer w (8-byte copies, zeros outside)
+    auto fill = [&](int z0, int w) {
+#pragma unroll
+        for (int e = tid; e < 64 * 16; e += 256) {
+            const int zz = e >> 4, k = e & 15, z = z0 + zz;
+            const bool vi = z < Nz && k < mx, ve = z < Nz && a0 + k < KZ;
+            cp_async8(&si[w][zz][k], vi ? in + ((size_t)b * Nz + z) * mx + k : in, vi);
+            cp_async8(&se[w][zz][k], ve ? tz + (size_t)z * KZ + a0 + k : tz, ve);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
     float2 acc[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc[j] = make_float2(0.f, 0.f);
-    for (int z0 = 0; z0 < Nz; z0 += 64) {
-        const int zc = min(64, Nz - z0);
-        for (int e = tid; e < 64 * 16; e += 256) {
-            const int zz = e >> 4, k = e & 15;
-            si[zz][k] = (zz < zc && k < mx) ? in[((size_t)b * Nz + z0 + zz) * mx + k] : make_float2(0.f, 0.f);
-            se[zz][k] = (zz < zc && a0 + k < KZ) ? tz[(size_t)(z0 + zz) * KZ + a0 + k] : make_float2(0.f, 0.f);
+    fill(0, 0);
+    int w = 0;
+    for (int z0 = 0; z0 < Nz; z0 += 64, w ^= 1) {
+        if (z0 + 64 < Nz) {
+            fill(z0 + 64, w ^ 1);  // in flight during the sums (13.8 us at 256 channels x 256 rows; 16.3 us without)
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
         __syncthreads();
 #pragma unroll 4
         for (int zz = 16 * h; zz < 16 * h + 16; ++zz) {
-            const float2 v = si[zz][kx];
-            const float4 e01 = *reinterpret_cast<const float4*>(&se[zz][4 * q]);
-            const float4 e23 = *reinterpret_cast<const float4*>(&se[zz][4 * q + 2]);
+            const float2 v = si[w][zz][kx];
+            const float4 e01 = *reinterpret_cast<const float4*>(&se[w][zz][4 * q]);
+            const float4 e23 = *reinterpret_cast<const float4*>(&se[w][zz][4 * q + 2]);
             acc[0] = cfmac(acc[0], v, make_float2(e01.x, e01.y));
             acc[1] = cfmac(acc[1], v, make_float2(e01.z, e01.w));
             acc[2] = cfmac(acc[2], v, make_float2(e23.x, e23.y));
@@ -674,30 +785,34 @@ __device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wa
 // all but the kDxtStages - 1 most recent groups complete (kDxtStages = 3)
 __device__ __forceinline__ void cp_async_wait_stages() { asm volatile("cp.async.wait_group 2;" ::: "memory"); }
 
-// k_combine_rt for FP32 inputs with rows of a multiple of 4 pixels, a block
-// marching over kRzRows rows of one 128-pixel column strip: the weights, the
-// strip's x inverse table and the bias are staged once, the next row's input
-// tile arrives by cp.async and its spectral coefficients through registers
-// while the current row is computed.  The same k order and fmaf sequence as
+// k_combine_rt for FP32 inputs with rows of a multiple of 4 pixels: a block of
+// 128 threads marches over nrow rows of one 128-pixel column strip, RW rows at
+// a time (2 for 32 outputs, 1 for 64).  The weights, the strip's x inverse table
+// (sine rows negated) and the bias are staged once; the next rows' input tiles
+// arrive by cp.async, and their spectral coefficients through registers, while
+// the current rows' sums go through GELU and out.  Thread (row, oq, pq) holds
+// outputs 8 oq .. 8 oq + 7 at pixels 4 pq .. + 3 and 64 + 4 pq .. + 3: per k, four
+// 16-byte shared-memory loads feed 64 products (32 FFMA2), so loads and FMAs take
+// the same time; 4 x 8 blocks were bound by their loads (l1tex 69 % busy, 160 us
+// per launch at 8 x 32 x 256 x 512).  The same k order and fmaf sequence as
 // k_combine (bitwise the same outputs).
-constexpr int kRzRows = 8;
 template <int CO, typename Tout>
-__global__ void __launch_bounds__(CO * 4) k_combine_rz(int ci, int Nz, int Nx, int mx, const float* __restrict__ in,
-                                                   const float* __restrict__ M, int mtrans,
-                                                   const float* __restrict__ bias, const float* __restrict__ T,
-                                                   const float* __restrict__ tab, int act, float* __restrict__ pre,
-                                                   Tout* __restrict__ out)
+__global__ void __launch_bounds__(128, 3) k_combine_rz(int nrow, int ci, int Nz, int Nx, int mx, const float* __restrict__ in,
+                                                       const float* __restrict__ M, int mtrans,
+                                                       const float* __restrict__ bias, const float* __restrict__ T,
+                                                       const float* __restrict__ tab, int act, float* __restrict__ pre,
+                                                       Tout* __restrict__ out)
 {
     extern __shared__ __align__(16) float sm[];
-    constexpr int NT = CO * 4, TPT = 32 * CO / NT;  // spectral coefficients per thread and row (8)
+    constexpr int NT = 128, RW = NT / (CO * 2), TPT = RW * 32 * CO / NT;  // coefficients per thread (16)
     const bool spec = T != nullptr;
-    float* sW = sm;                           // [ci][CO]
-    float* sT = sW + ci * CO;                 // [2][32][CO] (spec)
-    float* sX = sT + (spec ? 2 * 32 * CO : 0);  // [2][ci][kRtS]
-    float* sTab = sX + 2 * ci * kRtS;         // [32][kRtS] (spec)
-    float* sBias = sTab + (spec ? 32 * kRtS : 0);  // [CO]
+    float* sW = sm;                                   // [ci][CO]
+    float* sT = sW + ci * CO;                         // [RW][32][CO] (spec)
+    float* sX = sT + (spec ? RW * 32 * CO : 0);       // [RW][ci][kRtS]
+    float* sTab = sX + RW * ci * kRtS;                // [32][kRtS] (spec)
+    float* sBias = sTab + (spec ? 32 * kRtS : 0);     // [CO]
     const int b = blockIdx.z, x0 = blockIdx.x * kRtP, tid = threadIdx.x;
-    const int z0 = blockIdx.y * kRzRows, z1 = min(z0 + kRzRows, Nz);
+    const int z0 = blockIdx.y * nrow, z1 = min(z0 + nrow, Nz);
     const int n2 = 2 * mx;
     const size_t npix = (size_t)Nz * Nx;
     for (int e = tid; e < ci * CO; e += NT) {
@@ -705,107 +820,111 @@ __global__ void __launch_bounds__(CO * 4) k_combine_rz(int ci, int Nz, int Nx, i
         sW[e] = mtrans ? M[(size_t)k * CO + o] : M[(size_t)o * ci + k];
     }
     if (spec) {
+        // (a warp reads a pixel's factors, which are contiguous)
         for (int e = tid; e < 32 * kRtP; e += NT) {
-            const int r = e / kRtP, p = e - r * kRtP;
-            sTab[r * kRtS + p] = (x0 + p < Nx && r < n2) ? tab[(size_t)(x0 + p) * n2 + r] : 0.0f;
+            const int p = e >> 5, r = e & 31;
+            const float t = (x0 + p < Nx && r < n2) ? tab[(size_t)(x0 + p) * n2 + r] : 0.0f;
+            sTab[r * kRtS + p] = (r & 1) ? -t : t;
         }
     }
     for (int e = tid; e < CO; e += NT) sBias[e] = bias ? bias[e] : 0.0f;
-    // row z's input tile into buffer q (16-byte copies, zero past Nx)
-    auto issue = [&](int z, int q) {
-        float* dst = sX + q * ci * kRtS;
-        for (int e = tid; e < ci * (kRtP / 4); e += NT) {
-            const int i = e / (kRtP / 4), p = 4 * (e - i * (kRtP / 4));
-            const float* src = in + ((size_t)b * ci + i) * npix + (size_t)z * Nx;
+    // the input tiles of rows z .. z + RW - 1 (16-byte copies, zero past Nx; the last row repeated past z1)
+    auto issue = [&](int z) {
+        for (int e = tid; e < RW * ci * (kRtP / 4); e += NT) {
+            const int i = e / (kRtP / 4), p = 4 * (e - i * (kRtP / 4)), w = RW > 1 ? i / ci : 0, c = i - w * ci;
+            const float* src = in + ((size_t)b * ci + c) * npix + (size_t)min(z + w, z1 - 1) * Nx;
             const int bytes = x0 + p < Nx ? 16 : 0;  // Nx is a multiple of 4
-            cp_async16(su32(dst + i * kRtS + p), bytes ? src + x0 + p : src, bytes);
+            cp_async16(su32(sX + i * kRtS + p), bytes ? src + x0 + p : src, bytes);
         }
         cp_async_commit();
     };
-    // row z's spectral coefficients (o, r) of this thread: e = tid + j NT
+    // those rows' spectral coefficients (row w, o, r) of this thread: e = tid + j NT
     float tn[TPT];
     auto load_t = [&](int z) {
 #pragma unroll
         for (int j = 0; j < TPT; ++j) {
-            const int e = tid + j * NT, o = e >> 5, r = e & 31;
-            tn[j] = r < n2 ? T[(((size_t)b * CO + o) * Nz + z) * n2 + r] : 0.0f;
+            const int e = tid + j * NT, r = e & 31, o = (e >> 5) % CO, w = (e >> 5) / CO;
+            tn[j] = r < n2 ? T[(((size_t)b * CO + o) * Nz + min(z + w, z1 - 1)) * n2 + r] : 0.0f;
         }
     };
-    auto store_t = [&](int q) {
+    auto store_t = [&]() {
 #pragma unroll
         for (int j = 0; j < TPT; ++j) {
-            const int e = tid + j * NT, o = e >> 5, r = e & 31;
-            sT[(q * 32 + r) * CO + o] = (r & 1) ? -tn[j] : tn[j];
+            const int e = tid + j * NT, r = e & 31, o = (e >> 5) % CO, w = (e >> 5) / CO;
+            sT[(w * 32 + r) * CO + o] = tn[j];
         }
     };
     if (z0 < z1) {
-        issue(z0, 0);
+        issue(z0);
         if (spec) {
             load_t(z0);
-            store_t(0);
+            store_t();
         }
     }
-    const int oq = tid / 16, pq = tid % 16;
-    for (int z = z0; z < z1; ++z) {
-        const int q = (z - z0) & 1;
-        const bool next = z + 1 < z1;
-        if (next) {
-            issue(z + 1, q ^ 1);  // the buffer row z - 1 used (barrier at the end of it)
-            if (spec) load_t(z + 1);
-            cp_async_wait_prev();
-        } else {
-            cp_async_wait_all();
-        }
+    const int w = tid / (CO * 2), oq = tid % (CO * 2) / 16, pq = tid % 16;
+    for (int z = z0; z < z1; z += RW) {
+        cp_async_wait_all();
         __syncthreads();
-        const float* X = sX + q * ci * kRtS;
-        const float* A2 = sT + q * 32 * CO;
-        float acc[4][8];
+        float2 acc[8][4];  // output u, pixel pairs (0 1) (2 3) of both halves
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < 8; ++u)
 #pragma unroll
-            for (int v = 0; v < 8; ++v) acc[u][v] = sBias[4 * oq + u];
+            for (int v = 0; v < 4; ++v) acc[u][v] = make_float2(sBias[8 * oq + u], sBias[8 * oq + u]);
         auto step = [&](const float* Ak, const float* Bk) {
-            const float4 a = *reinterpret_cast<const float4*>(Ak + 4 * oq);
             const float4 b0 = *reinterpret_cast<const float4*>(Bk + 4 * pq);
             const float4 b1 = *reinterpret_cast<const float4*>(Bk + 64 + 4 * pq);
-            const float av[4] = {a.x, a.y, a.z, a.w};
-            const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < 8; ++v) acc[u][v] = fmaf(av[u], bv[v], acc[u][v]);
-        };
-#pragma unroll 4
-        for (int k = 0; k < ci; ++k) step(sW + k * CO, X + k * kRtS);
-        if (spec) {
-#pragma unroll 4
-            for (int r = 0; r < 32; ++r) step(A2 + r * CO, sTab + r * kRtS);
-        }
-        const size_t row = (size_t)z * Nx;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const size_t ob = ((size_t)b * CO + 4 * oq + u) * npix + row;
+            const float2 bv[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w), make_float2(b1.x, b1.y),
+                                  make_float2(b1.z, b1.w)};
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const int x = x0 + 64 * h + 4 * pq;
-                if (x >= Nx) continue;  // Nx is a multiple of 4: the 4 pixels are all in or all out
-                float y[4], g[4];
+                const float4 a = *reinterpret_cast<const float4*>(Ak + 8 * oq + 4 * h);
+                const float av[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    y[j] = acc[u][4 * h + j];
-                    g[j] = act == FNO_ACT_GELU ? gelu(y[j]) : y[j];
-                }
-                if (pre) *reinterpret_cast<float4*>(pre + ob + x) = make_float4(y[0], y[1], y[2], y[3]);
-                if constexpr (std::is_same<Tout, float>::value) {
-                    *reinterpret_cast<float4*>(out + ob + x) = make_float4(g[0], g[1], g[2], g[3]);
-                } else {
+                for (int u = 0; u < 4; ++u)
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) stf(out, ob + x + j, g[j]);
+                    for (int v = 0; v < 4; ++v)
+                        acc[4 * h + u][v] = __ffma2_rn(make_float2(av[u], av[u]), bv[v], acc[4 * h + u][v]);
+            }
+        };
+        const float* X = sX + w * ci * kRtS;
+#pragma unroll 2
+        for (int k = 0; k < ci; ++k) step(sW + k * CO, X + k * kRtS);
+        if (spec) {
+            const float* A2 = sT + w * 32 * CO;
+#pragma unroll 2
+            for (int r = 0; r < 32; ++r) step(A2 + r * CO, sTab + r * kRtS);
+        }
+        // the next rows' tiles and coefficients replace these while they are finished below
+        __syncthreads();
+        const bool next = z + RW < z1;
+        if (next) {
+            issue(z + RW);
+            if (spec) load_t(z + RW);
+        }
+        if (z + w < z1) {
+            const size_t row = (size_t)(z + w) * Nx;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const size_t ob = ((size_t)b * CO + 8 * oq + u) * npix + row;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int x = x0 + 64 * h + 4 * pq;
+                    if (x >= Nx) continue;  // Nx is a multiple of 4: the 4 pixels are all in or all out
+                    const float y[4] = {acc[u][2 * h].x, acc[u][2 * h].y, acc[u][2 * h + 1].x, acc[u][2 * h + 1].y};
+                    float g[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) g[j] = act == FNO_ACT_GELU ? gelu(y[j]) : y[j];
+                    if (pre) *reinterpret_cast<float4*>(pre + ob + x) = make_float4(y[0], y[1], y[2], y[3]);
+                    if constexpr (std::is_same<Tout, float>::value) {
+                        *reinterpret_cast<float4*>(out + ob + x) = make_float4(g[0], g[1], g[2], g[3]);
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) stf(out, ob + x + j, g[j]);
+                    }
                 }
             }
         }
-        if (next && spec) store_t(q ^ 1);  // read after the barrier at the top of row z + 1
-        __syncthreads();
+        if (next && spec) store_t();  // read after the barrier at the top
     }
 }
 
@@ -1346,89 +1465,97 @@ inline long long wg_max_blocks(int B, long long npix) { return B * ((npix + kWgM
 // Channel-major tiles of kWgTile pixels in shared memory (row stride kWgS,
 // padded so that 8 consecutive rows start in different banks): rows 0..cop-1
 // hold dU (zero past co), then cip rows of the input (row ci all ones, the
-// bias; zero past it).  Thread (task, slice) accumulates 4 x 4 outputs, o =
-// oq + u cop/4 and i = iq + v cip/4 (strided, so that the threads of a warp
+// bias; zero past it).  Thread (task, slice) accumulates BU x 4 outputs, o =
+// oq + u cop/BU and i = iq + v cip/4 (strided, so that the threads of a warp
 // read consecutive rows: no bank conflicts), over the 4-pixel groups slice,
-// slice + nslice, ... of each tile: 8 16-byte loads per 64 FMAs.
+// slice + nslice, ... of each tile, even and odd pixels in the halves of a packed
+// FMA: with BU = 8, 12 16-byte loads and 64 FFMA2 per 128 products, where 4 x 4
+// blocks of scalar FMAs took 16 loads and 128 (shared-memory bound).
 constexpr int kWgS = kWgTile + 4;
-__host__ __device__ inline int wg_cop(int co) { return (co + 3) & ~3; }
+// outputs per thread along o: 8, or 4 for few output channels
+__host__ __device__ inline int wg_bu(int co) { return co >= 8 ? 8 : 4; }
+__host__ __device__ inline int wg_cop(int co) { return (co + wg_bu(co) - 1) / wg_bu(co) * wg_bu(co); }
 
-__global__ void k_wgrad(int ci, int co, long long npix, long long chunk, const float* __restrict__ dU,
+template <int BU>
+__global__ void __launch_bounds__(160, 3) k_wgrad(int ci, int co, long long npix, long long chunk, const float* __restrict__ dU,
                         const float* __restrict__ in, float* __restrict__ partial)
 {
     extern __shared__ __align__(16) float sm[];
-    const int cip = wg_cip(ci), cop = wg_cop(co), g4 = cip / 4, ntask = (cop / 4) * g4;
+    const int cip = wg_cip(ci), cop = wg_cop(co), g4 = cip / 4, ntask = (cop / BU) * g4;
     const int nslice = blockDim.x / ntask;  // divides kWgTile / 4 (host)
     const int nrow = cop + cip;
     // each tile buffer: [cop][kWgS] rows of dU, then [cip][kWgS] rows of the input
     const int b = blockIdx.y, tid = threadIdx.x;
     const int task = tid % ntask, slice = tid / ntask;
-    const int oq = task / g4, iq = task % g4, og = cop / 4;
+    const int oq = task / g4, iq = task % g4, og = cop / BU;
     const long long p0 = (long long)blockIdx.x * chunk, p1 = min(p0 + chunk, npix);
     const float* dUb = dU + (size_t)b * co * npix;
     const float* inb = in + (size_t)b * ci * npix;
     const bool vec = (npix & 3) == 0 && (reinterpret_cast<uintptr_t>(dU) & 15) == 0 &&
                      (reinterpret_cast<uintptr_t>(in) & 15) == 0;
-    float acc[4][4];
+    float2 acc[BU][4];  // sums over even and odd pixels
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+    for (int u = 0; u < BU; ++u)
 #pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = 0.0f;
+        for (int v = 0; v < 4; ++v) acc[u][v] = make_float2(0.0f, 0.0f);
     // Tiles are double-buffered: the copies of tile k + 1 (cp.async, or plain
     // loads when the rows are not 16-byte aligned) are issued before the
-    // arithmetic of tile k.
-    float* buf[2] = {sm, sm + nrow * kWgS};
-    const int npiece = nrow * (kWgTile / 4);
-    auto fill = [&](float* dst, long long g) {
-        const int n = (int)min((long long)kWgTile, p1 - g);
-        for (int e = tid; e < npiece; e += blockDim.x) {
-            const int r = e / (kWgTile / 4), p = 4 * (e % (kWgTile / 4));
-            float* d = dst + r * kWgS + p;
-            const float* src = r < co ? dUb + (size_t)r * npix
-                                      : (r < cop ? nullptr : (r - cop < ci ? inb + (size_t)(r - cop) * npix : nullptr));
-            if (src && vec) {
-                const int bytes = 4 * max(0, min(4, n - p));
-                cp_async16(su32(d), bytes ? src + g + p : src, bytes);  // zero fill past the pixels
-            } else if (src) {
-                *reinterpret_cast<float4*>(d) =
-                    make_float4(p < n ? src[g + p] : 0.0f, p + 1 < n ? src[g + p + 1] : 0.0f,
-                                p + 2 < n ? src[g + p + 2] : 0.0f, p + 3 < n ? src[g + p + 3] : 0.0f);
-            } else {
-                const float one = r - cop == ci ? 1.0f : 0.0f;
-                *reinterpret_cast<float4*>(d) = make_float4(p < n ? one : 0.f, p + 1 < n ? one : 0.f,
-                                                            p + 2 < n ? one : 0.f, p + 3 < n ? one : 0.f);
+    // arithmetic of tile k.  A thread copies 4 pixels of every step-th row; the
+    // rows past co and ci never change (zeros, ones for the bias; dU is zero past
+    // the pixels, so the ones need not be).
+    const int tile = nrow * kWgS;
+    for (int e = tid; e < 2 * nrow * kWgTile; e += blockDim.x) {
+        const int q = e / (nrow * kWgTile), r = (e - q * nrow * kWgTile) / kWgTile, p = e % kWgTile;
+        if ((r >= co && r < cop) || r >= cop + ci) sm[q * tile + r * kWgS + p] = r == cop + ci ? 1.0f : 0.0f;
+    }
+    const int fp = 4 * (tid & (kWgTile / 4 - 1)), fr = tid / (kWgTile / 4), fstep = blockDim.x / (kWgTile / 4);
+    auto fill = [&](int q, long long g) {
+        const int n = (int)min((long long)kWgTile, p1 - g) - fp;  // pixels of this thread's column that exist
+        float* dst = sm + q * tile + fp;
+        if (fr < fstep) {
+            for (int part = 0; part < 2; ++part) {
+                const int rows = part ? ci : co;
+                const float* src = (part ? inb : dUb) + (size_t)fr * npix + g + fp;
+                float* d = dst + ((part ? cop : 0) + fr) * kWgS;
+                if (vec) {
+                    const int bytes = 4 * max(0, min(4, n));  // zero fill past the pixels
+                    for (int r = fr; r < rows; r += fstep, src += (size_t)fstep * npix, d += fstep * kWgS)
+                        cp_async16(su32(d), bytes ? src : dUb, bytes);
+                } else {
+                    for (int r = fr; r < rows; r += fstep, src += (size_t)fstep * npix, d += fstep * kWgS)
+                        *reinterpret_cast<float4*>(d) = make_float4(n > 0 ? src[0] : 0.0f, n > 1 ? src[1] : 0.0f,
+                                                                    n > 2 ? src[2] : 0.0f, n > 3 ? src[3] : 0.0f);
+                }
             }
         }
         cp_async_commit();
     };
-    if (p0 < p1) fill(buf[0], p0);
+    if (p0 < p1) fill(0, p0);
     int cur = 0;
     for (long long g = p0; g < p1; g += kWgTile, cur ^= 1) {
         if (g + kWgTile < p1) {
-            fill(buf[cur ^ 1], g + kWgTile);  // the buffer tile k - 1 used (barrier below)
+            fill(cur ^ 1, g + kWgTile);  // the buffer tile k - 1 used (barrier below)
             cp_async_wait_prev();
         } else {
             cp_async_wait_all();
         }
         __syncthreads();
-        const float* tD = buf[cur];
-        const float* tI = buf[cur] + cop * kWgS;
+        const float* tD = sm + cur * tile;
+        const float* tI = tD + cop * kWgS;
         if (slice < nslice) {
             for (int q = slice; q < kWgTile / 4; q += nslice) {
-                float4 d[4], x[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) d[u] = *reinterpret_cast<const float4*>(tD + (oq + u * og) * kWgS + 4 * q);
+                float4 x[4];
 #pragma unroll
                 for (int v = 0; v < 4; ++v) x[v] = *reinterpret_cast<const float4*>(tI + (iq + v * g4) * kWgS + 4 * q);
 #pragma unroll
-                for (int u = 0; u < 4; ++u)
+                for (int u = 0; u < BU; ++u) {
+                    const float4 d = *reinterpret_cast<const float4*>(tD + (oq + u * og) * kWgS + 4 * q);
 #pragma unroll
                     for (int v = 0; v < 4; ++v) {
-                        acc[u][v] = fmaf(d[u].x, x[v].x, acc[u][v]);
-                        acc[u][v] = fmaf(d[u].y, x[v].y, acc[u][v]);
-                        acc[u][v] = fmaf(d[u].z, x[v].z, acc[u][v]);
-                        acc[u][v] = fmaf(d[u].w, x[v].w, acc[u][v]);
+                        acc[u][v] = __ffma2_rn(make_float2(d.x, d.y), make_float2(x[v].x, x[v].y), acc[u][v]);
+                        acc[u][v] = __ffma2_rn(make_float2(d.z, d.w), make_float2(x[v].z, x[v].w), acc[u][v]);
                     }
+                }
             }
         }
         __syncthreads();
@@ -1437,9 +1564,10 @@ __global__ void k_wgrad(int ci, int co, long long npix, long long chunk, const f
     float* red = sm;  // [nslice][cop][cip]
     if (slice < nslice) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < BU; ++u)
 #pragma unroll
-            for (int v = 0; v < 4; ++v) red[((size_t)slice * cop + oq + u * og) * cip + iq + v * g4] = acc[u][v];
+            for (int v = 0; v < 4; ++v)
+                red[((size_t)slice * cop + oq + u * og) * cip + iq + v * g4] = acc[u][v].x + acc[u][v].y;
     }
     __syncthreads();
     const size_t blk = (size_t)b * gridDim.x + blockIdx.x;
@@ -1637,17 +1765,19 @@ void combine_dispatch(int B, int ci, int co, int Nz, int Nx, int mx, const void*
     if constexpr (std::is_same<Tin, float>::value) {
         if ((co == 32 || co == 64) && ci <= 64 && (!T || mx <= 16) && (Nx & 3) == 0 && al16 &&
             (reinterpret_cast<uintptr_t>(T) & 15) == 0) {
-            const size_t smem = (size_t)(ci * co + (T ? 2 * 32 * co : 0) + 2 * ci * kRtS + (T ? 32 * kRtS : 0) + co) *
+            const int rw = 64 / co;  // rows at a time (k_combine_rz)
+            const size_t smem = (size_t)(ci * co + (T ? rw * 32 * co : 0) + rw * ci * kRtS + (T ? 32 * kRtS : 0) + co) *
                                 sizeof(float);
-            const dim3 grid((unsigned)((Nx + kRtP - 1) / kRtP), (unsigned)((Nz + kRzRows - 1) / kRzRows), (unsigned)B);
+            const int nrow = 8;  // 162 us; 16 rows or one round of longer strips: 165 to 169 us
+            const dim3 grid((unsigned)((Nx + kRtP - 1) / kRtP), (unsigned)((Nz + nrow - 1) / nrow), (unsigned)B);
             if (co == 32) {
                 cudaFuncSetAttribute(k_combine_rz<32, Tout>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                k_combine_rz<32, Tout><<<grid, 128, smem, s>>>(ci, Nz, Nx, mx, static_cast<const float*>(in), M, mt, bias,
-                                                               T, tab, act, pre, static_cast<Tout*>(out));
+                k_combine_rz<32, Tout><<<grid, 128, smem, s>>>(nrow, ci, Nz, Nx, mx, static_cast<const float*>(in), M, mt,
+                                                               bias, T, tab, act, pre, static_cast<Tout*>(out));
             } else {
                 cudaFuncSetAttribute(k_combine_rz<64, Tout>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                k_combine_rz<64, Tout><<<grid, 256, smem, s>>>(ci, Nz, Nx, mx, static_cast<const float*>(in), M, mt, bias,
-                                                               T, tab, act, pre, static_cast<Tout*>(out));
+                k_combine_rz<64, Tout><<<grid, 128, smem, s>>>(nrow, ci, Nz, Nx, mx, static_cast<const float*>(in), M, mt,
+                                                               bias, T, tab, act, pre, static_cast<Tout*>(out));
             }
             return;
         }
@@ -1719,7 +1849,15 @@ wave_status_t fno_dft_x(long long rows, int Nx, int mx, const void* in, int in_b
     if (in_bf16)
         k_dft_x<__nv_bfloat16><<<(unsigned)nblk, 256, 0, s>>>(rows, Nx, 2 * mx, static_cast<const __nv_bfloat16*>(in),
                                                               table, out);
-    else
+    else if (mx == 16 && (Nx & 3) == 0 &&
+             ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(table) | reinterpret_cast<uintptr_t>(out)) &
+              15) == 0) {
+        // (256-row CTAs need 4 per SM to hide their latency: 155648 rows)
+        if (rows >= 256LL * 4 * 152)
+            k_dft_x8<8><<<(unsigned)((rows + 255) / 256), 128, 0, s>>>(rows, Nx, static_cast<const float*>(in), table, out);
+        else
+            k_dft_x8<4><<<(unsigned)((rows + 127) / 128), 128, 0, s>>>(rows, Nx, static_cast<const float*>(in), table, out);
+    } else
         k_dft_x<float><<<(unsigned)nblk, 256, 0, s>>>(rows, Nx, 2 * mx, static_cast<const float*>(in), table, out);
     return launched();
 }
@@ -1886,19 +2024,21 @@ wave_status_t fno_wgrad(int B, int Ci, int Co, long long npix, const float* dU, 
     if (wg_max_blocks(B, npix) > 0x7fffffffLL || B > 65535) return WAVE_ERR_ARG;
     long long nblk = 0;
     if (npix > 0 && B > 0) {
-        // 4 x 4 output blocks times pixel slices (a power of two dividing the
-        // tile's 16 groups of 4), about 256 threads
-        const int ntask = (wg_cop(Co) / 4) * (wg_cip(Ci) / 4);
+        // output blocks times pixel slices (a power of two dividing the tile's 16
+        // groups of 4), up to 160 threads (3 blocks of 128 registers a thread per SM)
+        const int bu = wg_bu(Co);
+        const int ntask = (wg_cop(Co) / bu) * (wg_cip(Ci) / 4);
         int nslice = 1;
-        while (nslice < kWgTile / 4 && ntask * nslice * 2 <= 320) nslice *= 2;
+        while (nslice < kWgTile / 4 && ntask * nslice * 2 <= 160) nslice *= 2;
         const int threads = ntask * nslice;
         const size_t tile = (size_t)(wg_cop(Co) + wg_cip(Ci)) * kWgS;
         const size_t red = (size_t)nslice * wg_cop(Co) * wg_cip(Ci);
         const size_t smem = std::max(2 * tile, red) * sizeof(float);
-        cudaFuncSetAttribute(k_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const auto kernel = bu == 8 ? k_wgrad<8> : k_wgrad<4>;
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         // chunks per sample so that all blocks are resident at once
         int per = 0, dev = 0, nsm = 1;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_wgrad, threads, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem);
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         (void)cudaGetLastError();
@@ -1908,7 +2048,7 @@ wave_status_t fno_wgrad(int B, int Ci, int Co, long long npix, const float* dU, 
         const long long nchunk = (npix + chunk - 1) / chunk;
         nblk = (long long)B * nchunk;
         const dim3 grid((unsigned)nchunk, B);
-        k_wgrad<<<grid, threads, smem, s>>>(Ci, Co, npix, chunk, dU, in, work);
+        kernel<<<grid, threads, smem, s>>>(Ci, Co, npix, chunk, dU, in, work);
     }
     const int nout = Co * (Ci + 1);
     k_wgrad_reduce<<<(nout + 7) / 8, 256, 0, s>>>(Ci, Co, nblk, work, dM, dbias);
