@@ -82,6 +82,25 @@ __device__ __forceinline__ void cluster_wait()
 {
     asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
+// Bounded wait (as mbar_wait) on a phase that other CTAs' st.async complete.  Their
+// complete_tx releases at cluster scope; try_wait without a scope acquires at CTA
+// scope only, which does not synchronise with it: neither the halo rows nor the
+// order of a neighbour's reads before this CTA's next writes would be guaranteed.
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* b, uint32_t parity)
+{
+    for (int it = 0; it < (1 << 22); ++it) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(smem_u32(b)), "r"(parity)
+            : "memory");
+        if (ok) return true;
+    }
+    return false;
+}
 __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes)
 {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
@@ -521,7 +540,7 @@ __global__ void __launch_bounds__(NT, 1) k_chip2d(const __grid_constant__ ChipAr
         if (a.C > 1) {
             if (tid == 0) mbar_expect_tx(&halo[1 - (i & 1)], halo_bytes);
             // (a thread whose wait gives up records it and goes on: every barrier below stays uniform)
-            if (border && i > 0 && alive && !mbar_wait(&halo[i & 1], (uint32_t)((i - 1) >> 1) & 1u)) {
+            if (border && i > 0 && alive && !mbar_wait_cluster(&halo[i & 1], (uint32_t)((i - 1) >> 1) & 1u)) {
                 alive = false;
                 atomicOr(a.err, kErrTimeout);
             }
@@ -571,7 +590,7 @@ __global__ void __launch_bounds__(NT, 1) k_chip2d(const __grid_constant__ ChipAr
     }
     if (a.C > 1) {
         // the last rows sent to this CTA have landed, and all of the cluster is here, before any CTA leaves
-        if (tid == 0 && alive && a.nsteps > 0 && !mbar_wait(&halo[a.nsteps & 1], (uint32_t)((a.nsteps - 1) >> 1) & 1u))
+        if (tid == 0 && alive && a.nsteps > 0 && !mbar_wait_cluster(&halo[a.nsteps & 1], (uint32_t)((a.nsteps - 1) >> 1) & 1u))
             atomicOr(a.err, kErrTimeout);
         cluster_arrive();
         cluster_wait();

@@ -1,0 +1,23 @@
+"""What the on-chip time loop's source has to say about waits between CTAs: such a
+mistake need not show in results, and is not provoked on a GPU."""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2304_05592_gb300", "csrc")
+
+
+@pytest.fixture(scope="module")
+def chip():
+    text = open(os.path.join(CSRC, "step2d_chip.cu")).read()
+    return re.sub(r"//[^\n]*", "", text)  # (no string holds a //)
+
+
+def test_halo_waits_acquire_at_cluster_scope(chip):
+    # the halo rows come from other CTAs' st.async, released at cluster scope
+    assert "st.async" in chip
+    waits = re.findall(r"\b(mbar_\w*(?:wait|try)\w*)\s*\(\s*&halo", chip)
+    assert len(waits) >= 2 and set(waits) == {"mbar_wait_cluster"}, waits
+    forms = re.findall(r"mbarrier\.(?:try_wait|test_wait)[\w.:]*", chip)
+    assert forms and all(".acquire.cluster" in f for f in forms), forms
