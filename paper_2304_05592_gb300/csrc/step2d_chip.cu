@@ -538,7 +538,8 @@ __global__ void __launch_bounds__(NT, 1) k_chip2d(const __grid_constant__ ChipAr
             for (int t = t0; t < tg.n; t += blockDim.x) row[tg.ref[t]] = tg.fac[t] * lev[tg.off[t]];
         }
         if (a.C > 1) {
-            if (tid == 0) mbar_expect_tx(&halo[1 - (i & 1)], halo_bytes);
+            // (after a wait that gave up this barrier's last phase may be open still: no second arrival then)
+            if (tid == 0 && alive) mbar_expect_tx(&halo[1 - (i & 1)], halo_bytes);
             // (a thread whose wait gives up records it and goes on: every barrier below stays uniform)
             if (border && i > 0 && alive && !mbar_wait_cluster(&halo[i & 1], (uint32_t)((i - 1) >> 1) & 1u)) {
                 alive = false;
@@ -590,10 +591,17 @@ __global__ void __launch_bounds__(NT, 1) k_chip2d(const __grid_constant__ ChipAr
     }
     if (a.C > 1) {
         // the last rows sent to this CTA have landed, and all of the cluster is here, before any CTA leaves
-        if (tid == 0 && alive && a.nsteps > 0 && !mbar_wait_cluster(&halo[a.nsteps & 1], (uint32_t)((a.nsteps - 1) >> 1) & 1u))
+        if (tid == 0 && alive && a.nsteps > 0 && !mbar_wait_cluster(&halo[a.nsteps & 1], (uint32_t)((a.nsteps - 1) >> 1) & 1u)) {
+            alive = false;
             atomicOr(a.err, kErrTimeout);
+        }
         cluster_arrive();
         cluster_wait();
+        // every CTA has sent its rows by now: one that gave a wait up stays (bounded again) until
+        // those on their way to it have landed
+        if (tid == 0 && !alive)
+            for (int n = a.nsteps; n > 0 && n > a.nsteps - 2; --n)
+                mbar_wait_cluster(&halo[n & 1], (uint32_t)((n - 1) >> 1) & 1u);
     }
     const int nl = ADJ ? a.first - a.nsteps : a.first + a.nsteps;  // the index of the next step
     if (tg.n > 0 && a.nsteps > 0 && (ADJ || nl - 1 >= a.rec_from)) {
