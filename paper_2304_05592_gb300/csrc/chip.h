@@ -60,4 +60,16 @@ ChipPlan chip_plan(const Dims& d, const Tiling& t, int nshot, int mode, const Ho
 void launch_chip_tap_gradient(const TapList& l, int nt, long long cell, const float* tacc, float* g, cudaStream_t s);
 cudaError_t launch_chip(const ChipPlan& p, ChipArgs& a, int nshot, cudaStream_t s);
 
+// Restricts chip_plan to one shape (index into kShapes, -1: any) and one cluster
+// size (0: any), so that tests reach every instantiation: the estimate takes one per
+// problem.  refuse: launches ask for more shared memory than there is, which the CUDA
+// runtime refuses on the host, so that tests see how a failed launch is reported.  Per
+// host thread; nothing else sets it.
+struct ChipForce {
+    int shape = -1, C = 0;
+    bool refuse = false;
+};
+
 }  // namespace wave
+
+extern "C" int wave_chip_force(int shape, int clusters, int refuse);  // returns the number of shapes

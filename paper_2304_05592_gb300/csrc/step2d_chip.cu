@@ -778,6 +778,8 @@ bool one_sided(int Nz, int C, int NC)
 
 }  // namespace
 
+thread_local ChipForce t_force;  // of calls from this host thread; set by tests only
+
 ChipPlan chip_plan(const Dims& d, const Tiling& t, int nshot, int mode, const HostTaps& inj, const HostTaps& gat)
 {
     ChipPlan best;
@@ -789,7 +791,9 @@ ChipPlan chip_plan(const Dims& d, const Tiling& t, int nshot, int mode, const Ho
     for (int C = 1; C <= kMaxCluster; ++C) {
         const int R = (d.Nz + C - 1) / C;
         if (C > 1 && d.Nz / C < 4) break;  // a strip feeds its neighbours' 4-row halos
+        if (t_force.C && C != t_force.C) continue;
         for (int k = 0; k < kShapeCount; ++k) {
+            if (t_force.shape >= 0 && k != t_force.shape) continue;
             const int NT = kShapes[k].NT[mode];
             const int NC = (R + kShapes[k].RB - 1) / kShapes[k].RB;
             const int threads = (NC * Q + 31) / 32 * 32;
@@ -846,6 +850,7 @@ cudaError_t launch_chip(const ChipPlan& p, ChipArgs& a, int nshot, cudaStream_t 
     cudaLaunchAttribute at[1];
     cudaLaunchConfig_t cfg = chip_config(p, nshot, s, at);
     count_step_launch();
+    if (t_force.refuse) cfg.dynamicSmemBytes = (size_t)1 << 30;
     cudaEvent_t stop;
     const bool timed = profile_sample(p.mode >= kChipAdjoint, s, &stop, a.nsteps);
     const cudaError_t e = cudaLaunchKernelEx(&cfg, k, a);
@@ -861,3 +866,11 @@ void launch_chip_tap_gradient(const TapList& l, int nt, long long cell, const fl
 }
 
 }  // namespace wave
+
+extern "C" int wave_chip_force(int shape, int clusters, int refuse)
+{
+    wave::t_force.shape = shape;
+    wave::t_force.C = clusters;
+    wave::t_force.refuse = refuse != 0;
+    return wave::kShapeCount;
+}
