@@ -162,9 +162,9 @@ wave_status_t plan(const wave_grid_t* g, int op, int nshot, int nsrc, const floa
         L.iA0 = 0;
         L.nbuf = 2;
     } else if (op == 3) {
-        L.iW0 = 0;  // three background levels W0 W1 W2, then the scattered field A0 A1
-        L.iA0 = 3;
-        L.nbuf = 5;
+        L.iW0 = 0;  // the background levels, a third one in 3D, then the scattered field A0 A1
+        L.iA0 = L.d.ndim == 3 ? 3 : 2;
+        L.nbuf = L.iA0 + 2;
     } else {
         L.iW0 = 0;
         L.iA0 = 2;
@@ -646,6 +646,7 @@ public:
         const cudaError_t e = launch_chip(dir_ == 1 ? L.cf : L.ca, *a_, L.nshot, s);
         if (e != cudaSuccess) {
             note_cuda_error(e);
+            (void)cudaGetLastError();  // reported through failed(); the next call must not find it
             failed_ = true;
         }
         dir_ = 0;
@@ -1073,7 +1074,7 @@ wave_status_t wave_born(const wave_grid_t* grid, const float* vel, int nshot, in
     if ((st = setup(L, vel, s))) return st;
     launch_prep_dm(L.d, dm, L.kap, L.dmv, s);
     const size_t fb = L.field() * sizeof(float);
-    CK(cudaMemsetAsync(L.buf(0), 0, 5 * fb, s));
+    CK(cudaMemsetAsync(L.buf(0), 0, L.nbuf * fb, s));
     const size_t nrow = L.hr.idx.size();
     if (nrow) CK(cudaMemsetAsync(L.slots_rec, 0, nrow * sizeof(float), s));
     int dcur = L.iA0, dprev = L.iA0 + 1;
@@ -1190,8 +1191,11 @@ wave_status_t wave_autotune(const wave_grid_t* grid, const float* vel, int nshot
                 }
                 m = std::max(1, std::min(16 * nstep, L.d.nt - 1));
             }
-            if (make_maps(L)) continue;
-            auto run = [&](int n_steps) {
+            if (make_maps(L)) {
+                L.cf = L.ca = ChipPlan();
+                continue;
+            }
+            auto run = [&](int n_steps) {  // false: the loop could not be launched
                 if (L.cf.C || L.ca.C) {
                     StepQueue q(L, wavelet, L.dsyn, nullptr, false, s);
                     for (int k = 0; k < n_steps; ++k) {
@@ -1200,7 +1204,7 @@ wave_status_t wave_autotune(const wave_grid_t* grid, const float* vel, int nshot
                         else q.adj(L.iA0 + b, L.iA0 + 1 - b, L.d.nt - 1 - k, L.iW0, -1);
                     }
                     q.flush();
-                    return;
+                    return !q.failed();
                 }
                 for (int k = 0; k < n_steps; ++k) {
                     const int n = k % std::max(1, L.d.nt - 1);
@@ -1209,10 +1213,11 @@ wave_status_t wave_autotune(const wave_grid_t* grid, const float* vel, int nshot
                     else adj_step(L, L.iA0 + (k & 1), L.iA0 + 1 - (k & 1), std::max(1, n), L.dsyn, nullptr, false,
                                   L.iW0, -1, s);
                 }
+                return true;
             };
-            run(std::min(2, m));
+            bool ran = run(std::min(2, m));
             cudaEventRecord(e0, s);
-            run(m);
+            ran = run(m) && ran;
             cudaEventRecord(e1, s);
             if (cudaEventSynchronize(e1) != cudaSuccess) {
                 cudaEventDestroy(e0);
@@ -1224,7 +1229,7 @@ wave_status_t wave_autotune(const wave_grid_t* grid, const float* vel, int nshot
             cudaEventElapsedTime(&ms, e0, e1);
             ms *= (float)nstep / m;
             L.cf = L.ca = ChipPlan();
-            if (ms < best[which]) {
+            if (ran && ms < best[which]) {
                 best[which] = ms;
                 pick[which] = v;
             }
