@@ -162,9 +162,9 @@ wave_status_t plan(const wave_grid_t* g, int op, int nshot, int nsrc, const floa
         L.iA0 = 0;
         L.nbuf = 2;
     } else if (op == 3) {
-        L.iW0 = 0;  // three background levels W0 W1 W2, then the scattered field A0 A1
-        L.iA0 = 3;
-        L.nbuf = 5;
+        L.iW0 = 0;  // the background levels, a third one in 3D, then the scattered field A0 A1
+        L.iA0 = L.d.ndim == 3 ? 3 : 2;
+        L.nbuf = L.iA0 + 2;
     } else {
         L.iW0 = 0;
         L.iA0 = 2;
@@ -1074,7 +1074,7 @@ wave_status_t wave_born(const wave_grid_t* grid, const float* vel, int nshot, in
     if ((st = setup(L, vel, s))) return st;
     launch_prep_dm(L.d, dm, L.kap, L.dmv, s);
     const size_t fb = L.field() * sizeof(float);
-    CK(cudaMemsetAsync(L.buf(0), 0, 5 * fb, s));
+    CK(cudaMemsetAsync(L.buf(0), 0, L.nbuf * fb, s));
     const size_t nrow = L.hr.idx.size();
     if (nrow) CK(cudaMemsetAsync(L.slots_rec, 0, nrow * sizeof(float), s));
     int dcur = L.iA0, dprev = L.iA0 + 1;

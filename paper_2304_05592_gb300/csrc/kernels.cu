@@ -159,8 +159,6 @@ __global__ void __launch_bounds__(32 * BZ, 1024 / (32 * BZ)) k_step2d(const Step
         const long long off = (long long)gz * a.P + gx;
         const int dz = sponge_depth(gz, a.nb, a.nz);
         float out[4], cen[4], um[4], uf[4] = {0.f, 0.f, 0.f, 0.f};
-        float bsrc[4] = {0.f, 0.f, 0.f, 0.f};
-        if (a.dmv) born_source(a, so, off, bsrc);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int dd = max(sponge_depth(gx + i, a.nb, a.nx), dz);
@@ -168,7 +166,7 @@ __global__ void __launch_bounds__(32 * BZ, 1024 / (32 * BZ)) k_step2d(const Step
             const float eps = kap * a.ceps * (float)(dd * dd);
             cen[i] = w[i + 4];
             um[i] = f4(uo[rr], i);
-            out[i] = leap1(cen[i], um[i], lap[i], kap, eps, rcp_sponge(1.0f + eps), bsrc[i]);
+            out[i] = leap1(cen[i], um[i], lap[i], kap, eps, rcp_sponge(1.0f + eps), 0.0f);
         }
         float4 gv = make_float4(0.f, 0.f, 0.f, 0.f);
         if (imaging) {
