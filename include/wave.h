@@ -337,15 +337,16 @@ wave_status_t wave_checkpoint_schedule(int nt, int nsnap, long long* fwd_steps, 
 
 /* Measurement support (no counterpart in the paper).
  * wave_launch_count: number of kernels this library has launched so far in
- * the process.  wave_profile_start(every): from now on, bracket every
- * `every`-th stencil time-step launch with two CUDA events on its stream
- * (at most 8192 samples); every = 0 instead brackets each run of consecutive
- * step launches of one kind (forward or adjoint) on one stream, which keeps
- * the overlap between consecutive launches inside a run (at most 16384 runs;
- * a run ends at a change of kind or stream or at another library kernel).
- * wave_profile_stop: stops sampling, waits for the sampled events and returns
- * the summed milliseconds and the number of forward and adjoint step
- * launches they cover (any pointer may be NULL). */
+ * the process.  wave_profile_start(every): from now on, bracket the launch
+ * that makes every `every`-th stencil time step with two CUDA events on its
+ * stream (at most 8192 samples; the first step counts, and a launch of the
+ * on-chip 2D loop makes many steps); every = 0 instead brackets each run of
+ * consecutive step launches of one kind (forward or adjoint) on one stream,
+ * which keeps the overlap between consecutive launches inside a run (at most
+ * 16384 runs; a run ends at a change of kind or stream or at another library
+ * kernel).  wave_profile_stop: stops sampling, waits for the sampled events and
+ * returns the summed milliseconds and the number of forward and adjoint time
+ * steps that the sampled launches made (any pointer may be NULL). */
 long long wave_launch_count(void);
 wave_status_t wave_profile_start(int every);
 wave_status_t wave_profile_stop(double* fwd_ms, long long* fwd_n, double* adj_ms, long long* adj_n);

@@ -20,7 +20,7 @@ std::atomic<long long> g_launches{0};
 std::mutex g_mu;
 bool g_on = false;
 int g_every = 1;
-long long g_seen = 0;
+long long g_seen = 0;  // time steps since wave_profile_start
 std::vector<Sample> g_samples;  // recorded during the current region
 std::vector<cudaEvent_t> g_pool;
 size_t g_pool_next = 0;
@@ -96,8 +96,10 @@ bool profile_sample(bool adjoint, cudaStream_t s, cudaEvent_t* stop, int steps)
         g_run_stream = s;
         return false;
     }
-    const bool take = (g_seen++ % g_every) == 0 && g_samples.size() < kMaxSamples;
-    if (!take) return false;
+    // every g_every-th step is due, and a launch that holds a due step is sampled
+    const long long past = g_seen % g_every;  // steps since the last due one
+    g_seen += steps;
+    if ((past > 0 && past + steps <= g_every) || g_samples.size() >= kMaxSamples) return false;
     Sample smp;
     smp.start = take_event();
     smp.stop = take_event();

@@ -418,15 +418,15 @@ def wave_launch_count() -> int:
 
 
 def wave_profile_start(every: int = 1) -> None:
-    """Bracket every `every`-th stencil step launch with CUDA events (every = 0:
-    each run of consecutive step launches of one kind, overlap kept)."""
+    """Bracket the launch of every `every`-th stencil time step with CUDA events (every
+    = 0: each run of consecutive step launches of one kind, overlap kept)."""
     st = _lib().wave_profile_start(int(every))
     if st:
         raise WaveError(st, "wave_profile_start")
 
 
 def wave_profile_stop():
-    """(forward ms, forward samples, adjoint ms, adjoint samples) since start."""
+    """(forward ms, forward time steps sampled, adjoint ms, adjoint time steps) since start."""
     f, a = ctypes.c_double(0), ctypes.c_double(0)
     nf, na = ctypes.c_longlong(0), ctypes.c_longlong(0)
     st = _lib().wave_profile_stop(ctypes.byref(f), ctypes.byref(nf), ctypes.byref(a), ctypes.byref(na))

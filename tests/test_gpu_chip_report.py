@@ -1,5 +1,6 @@
-"""What the on-chip 2D time loop reports of launches that CUDA refuses (on the host: a
-request for more shared memory than there is)."""
+"""What the on-chip 2D time loop reports: launches that CUDA refuses (on the host: a
+request for more shared memory than there is), and profile samples of launches that
+hold many time steps."""
 import ctypes
 
 import numpy as np
@@ -70,3 +71,16 @@ def test_autotune_does_not_pick_a_loop_that_cannot_be_launched():
     _refuse(False)
     again = wave.wave_autotune(g, v, p.src, q, p.rec, steps=4)
     assert picked[0] != last[0] and picked[1] != last[1], (picked, again)
+
+
+@pytest.mark.parametrize("every", [1, 10, 60])
+def test_profile_samples_every_nth_step(every):
+    """`every` counts time steps: a launch that holds many of them is sampled if one of them is due.  80
+    samples: 79 forward steps, then 79 adjoint steps."""
+    p, g, v, q, d = _case()
+    wave.wave_gradient(g, v, p.src, q, p.rec, d, store=wave.STORE_FP32)
+    wave.wave_profile_start(every)
+    wave.wave_gradient(g, v, p.src, q, p.rec, d, store=wave.STORE_FP32)
+    fms, fn, ams, an = wave.wave_profile_stop()
+    assert fn == p.nt - 1 and fms > 0.0
+    assert an == p.nt - 1 and ams > 0.0
