@@ -123,7 +123,8 @@ struct StepArgs {
     float* gacc;         // [nshot][cell]
     int* err;
     // Born scattering source: unew gets -dmv .* (bs_a - 2 bs_b + bs_c) / (1 + eps)
-    // added, dmv = Extend(dm) v^2 (kind 0 2D kernel and the 3D kernel only)
+    // added, dmv = Extend(dm) v^2 (3D z-march; the 2D Born step takes dmv alone and
+    // has the background levels itself)
     const float* dmv;
     const float *bs_a, *bs_b, *bs_c;
     // pool indices of the same buffers for the TMA kernels (-1: none)
