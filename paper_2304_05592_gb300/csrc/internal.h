@@ -226,3 +226,6 @@ struct Schedule {
 Schedule make_schedule(int nt, int nsnap);
 
 }  // namespace wave
+
+// The choice of shot_group for tests (host only, no device work).
+extern "C" int wave_shot_group(const wave_grid_t* grid, int nshot, int adjoint, float* step_us);

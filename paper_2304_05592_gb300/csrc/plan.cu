@@ -62,13 +62,18 @@ int shot_group(const Dims& d, int nshot, bool adjoint, float* step_us)
     const float tiles = (float)((d.Nx + kTX - 1) / kTX) * ((d.Nz + 15) / 16);
     int best = 4;
     float least = 0.0f;
-    for (int k = 2; k >= 0; --k) {
+    for (int k = nshot > 1 ? 2 : 1; k >= 0; --k) {
         const int g = 1 << k;
-        const float n = tiles * ((nshot + g - 1) / g), *c = kChain[adjoint][k], *r = kRate[adjoint][k];
-        // (a group larger than the batch is as long as the batch)
-        const float chain = nshot < g ? kChain[adjoint][0][0] + (c[0] - kChain[adjoint][0][0]) * (nshot - 1) / (g - 1) : c[0];
-        const float t = std::max(chain + c[1] * n, nshot < g ? 0.0f : r[0] + r[1] * n);
-        if (k == 2 || t < least) {
+        const float n = tiles * ((nshot + g - 1) / g), *c = kChain[adjoint][k];
+        const auto rate = [&](int j) { return kRate[adjoint][j][0] + kRate[adjoint][j][1] * n; };
+        // a group larger than the batch is as long as the batch and does the work of a group of its size
+        float chain = c[0], gpu = rate(k);
+        if (nshot < g) {
+            chain = kChain[adjoint][0][0] + (c[0] - kChain[adjoint][0][0]) * (nshot - 1) / (g - 1);
+            gpu = nshot == 3 ? 0.5f * (rate(1) + rate(2)) : rate(nshot - 1);
+        }
+        const float t = std::max(chain + c[1] * n, gpu);
+        if (least == 0.0f || t < least) {
             best = g;
             least = t;
         }
@@ -373,3 +378,8 @@ Schedule make_schedule(int nt, int nsnap)
 }
 
 }  // namespace wave
+
+extern "C" int wave_shot_group(const wave_grid_t* g, int nshot, int adjoint, float* step_us)
+{
+    return wave::shot_group(wave::make_dims(*g), nshot, adjoint != 0, step_us);
+}
