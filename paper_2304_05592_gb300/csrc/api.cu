@@ -451,7 +451,7 @@ float launched_step_us(const Dims& d, int nshot, bool adjoint)
 void choose_chip(Layout& L)
 {
     if (L.d.ndim != 2 || L.op == 3) return;
-    auto pick = [&](int which, int& v, bool set, int mode, const HostTaps& inj, const HostTaps& gat) {
+    auto pick = [&](int which, int& v, bool set, int mode, HostTaps& inj, HostTaps& gat) {
         const bool asked = variant_info(which, v).kind == 8;
         ChipPlan p;
         if (asked || !set) p = chip_plan(L.d, L.t, L.nshot, mode, inj, gat);
@@ -462,7 +462,7 @@ void choose_chip(Layout& L)
         else if (asked) v = group_variant(which == 1, shot_group(L.d, L.nshot, which == 1, nullptr));
         return p;
     };
-    const HostTaps none;
+    HostTaps none;
     if (L.op == 0 || L.op == 2) L.cf = pick(0, L.t.vf, L.t.set_f, L.st16 ? kChipFwdBF16 : kChipForward, L.hs, L.hr);
     if (L.op == 1) L.ca = pick(1, L.t.va, L.t.set_a, kChipAdjoint, L.hr, L.hs);
     if (L.op == 2)
@@ -1174,7 +1174,7 @@ wave_status_t wave_autotune(const wave_grid_t* grid, const float* vel, int nshot
     float best[2] = {1e30f, 1e30f};
     int pick[2] = {current_variant(0), current_variant(1)};
     L.cf = L.ca = ChipPlan();
-    const HostTaps none;
+    HostTaps none;
     for (int which = 0; which < 2; ++which) {
         for (int v = 0; v < variant_count(which); ++v) {
             if (which == 0) L.t.vf = v;

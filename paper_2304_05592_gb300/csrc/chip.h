@@ -56,7 +56,8 @@ struct ChipPlan {
     size_t smem = 0;
     float step_us = 0.0f;  // estimated time of one step of all shots
 };
-ChipPlan chip_plan(const Dims& d, const Tiling& t, int nshot, int mode, const HostTaps& inj, const HostTaps& gat);
+// (inj and gat keep their taps per strip for the next plan of the call)
+ChipPlan chip_plan(const Dims& d, const Tiling& t, int nshot, int mode, HostTaps& inj, HostTaps& gat);
 void launch_chip_tap_gradient(const TapList& l, int nt, long long cell, const float* tacc, float* g, cudaStream_t s);
 cudaError_t launch_chip(const ChipPlan& p, ChipArgs& a, int nshot, cudaStream_t s);
 

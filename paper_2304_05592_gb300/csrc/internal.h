@@ -73,6 +73,9 @@ struct HostTaps {
     std::vector<float> w;
     int npts = 0;
     size_t ntap = 0, npt_start = 0;  // sizes of the tables, also when only counted
+    // per cluster size C of the on-chip loop: the most taps, and the most grid rows with
+    // taps, that any strip of any shot holds (filled when a plan first asks)
+    std::vector<int> strip_taps, strip_rows;
 };
 
 // Builds taps for nshot * npts points; WAVE_ERR_GEOMETRY for a point outside
