@@ -261,13 +261,6 @@ __device__ __forceinline__ void cp_async8(void* dst, const void* src, bool ok)
                  : "memory");
 }
 
-__device__ __forceinline__ void cp_async16z(void* dst, const void* src, bool ok)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
-                 "r"(ok ? 16 : 0)
-                 : "memory");
-}
-
 // out[b][a][kx] = sum_z in[b][z][kx] conj(E[z][a]); CTA per (b, 16 values of a).
 // Thread (h, q, kx) computes outputs (a0 + 4 q .. a0 + 4 q + 3, kx) over quarter h
 // of every 64-row chunk of z, so each in[z][kx] read from shared memory feeds
@@ -279,26 +272,14 @@ __global__ void __launch_bounds__(256) k_dft_z(int Nz, int KZ, int mx, const flo
     __shared__ float2 red[3][16][16];
     const int b = blockIdx.x, a0 = blockIdx.y * 16, tid = threadIdx.x;
     const int kx = tid & 15, q = (tid >> 4) & 3, h = tid >> 6;
-    // rows z0 .. z0 + 63 of the input and the table into buffer w, zeros outside: two modes per copy where
-    // rows begin at 16 bytes (KZ = 2 mz is even), else one
-    const bool pairs = (mx & 1) == 0 && ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(tz)) & 15) == 0;
+    // rows z0 .. z0 + 63 of the input and the table into buffer w (8-byte copies, zeros outside)
     auto fill = [&](int z0, int w) {
-        if (pairs) {
 #pragma unroll
-            for (int e = tid; e < 64 * 8; e += 256) {
-                const int zz = e >> 3, k = 2 * (e & 7), z = z0 + zz;
-                const bool vi = z < Nz && k < mx, ve = z < Nz && a0 + k < KZ;
-                cp_async16z(&si[w][zz][k], vi ? in + ((size_t)b * Nz + z) * mx + k : in, vi);
-                cp_async16z(&se[w][zz][k], ve ? tz + (size_t)z * KZ + a0 + k : tz, ve);
-            }
-        } else {
-#pragma unroll
-            for (int e = tid; e < 64 * 16; e += 256) {
-                const int zz = e >> 4, k = e & 15, z = z0 + zz;
-                const bool vi = z < Nz && k < mx, ve = z < Nz && a0 + k < KZ;
-                cp_async8(&si[w][zz][k], vi ? in + ((size_t)b * Nz + z) * mx + k : in, vi);
-                cp_async8(&se[w][zz][k], ve ? tz + (size_t)z * KZ + a0 + k : tz, ve);
-            }
+        for (int e = tid; e < 64 * 16; e += 256) {
+            const int zz = e >> 4, k = e & 15, z = z0 + zz;
+            const bool vi = z < Nz && k < mx, ve = z < Nz && a0 + k < KZ;
+            cp_async8(&si[w][zz][k], vi ? in + ((size_t)b * Nz + z) * mx + k : in, vi);
+            cp_async8(&se[w][zz][k], ve ? tz + (size_t)z * KZ + a0 + k : tz, ve);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
@@ -813,18 +794,18 @@ __device__ __forceinline__ void cp_async_wait_stages() { asm volatile("cp.async.
 // outputs 8 oq .. 8 oq + 7 at pixels 4 pq .. + 3 and 64 + 4 pq .. + 3: per k, four
 // 16-byte shared-memory loads feed 64 products (32 FFMA2), so loads and FMAs take
 // the same time; 4 x 8 blocks were bound by their loads (l1tex 69 % busy, 160 us
-// per launch at 8 x 32 x 256 x 512).  Without the spectral part 4 blocks fit an SM (91
-// us at that size, 96 with 3).  The same k order and fmaf sequence as k_combine
-// (bitwise the same outputs).
-template <int CO, bool SPEC, typename Tout>
-__global__ void __launch_bounds__(128, SPEC ? 3 : 4)
-    k_combine_rz(int nrow, int ci, int Nz, int Nx, int mx, const float* __restrict__ in, const float* __restrict__ M,
-                 int mtrans, const float* __restrict__ bias, const float* __restrict__ T, const float* __restrict__ tab,
-                 int act, float* __restrict__ pre, Tout* __restrict__ out)
+// per launch at 8 x 32 x 256 x 512).  The same k order and fmaf sequence as
+// k_combine (bitwise the same outputs).
+template <int CO, typename Tout>
+__global__ void __launch_bounds__(128, 3) k_combine_rz(int nrow, int ci, int Nz, int Nx, int mx, const float* __restrict__ in,
+                                                       const float* __restrict__ M, int mtrans,
+                                                       const float* __restrict__ bias, const float* __restrict__ T,
+                                                       const float* __restrict__ tab, int act, float* __restrict__ pre,
+                                                       Tout* __restrict__ out)
 {
     extern __shared__ __align__(16) float sm[];
     constexpr int NT = 128, RW = NT / (CO * 2), TPT = RW * 32 * CO / NT;  // coefficients per thread (16)
-    const bool spec = SPEC && T != nullptr;  // (a test at run time: without it the compiler schedules the sums 2 % slower)
+    const bool spec = T != nullptr;
     float* sW = sm;                                   // [ci][CO]
     float* sT = sW + ci * CO;                         // [RW][32][CO] (spec)
     float* sX = sT + (spec ? RW * 32 * CO : 0);       // [RW][ci][kRtS]
@@ -1491,15 +1472,16 @@ inline long long wg_max_blocks(int B, long long npix) { return B * ((npix + kWgM
 // FMA: with BU = 8, 12 16-byte loads and 64 FFMA2 per 128 products, where 4 x 4
 // blocks of scalar FMAs took 16 loads and 128 (shared-memory bound).
 constexpr int kWgS = kWgTile + 4;
-__host__ __device__ inline int wg_cop(int co, int bu) { return (co + bu - 1) / bu * bu; }
+// outputs per thread along o: 8, or 4 for few output channels
+__host__ __device__ inline int wg_bu(int co) { return co >= 8 ? 8 : 4; }
+__host__ __device__ inline int wg_cop(int co) { return (co + wg_bu(co) - 1) / wg_bu(co) * wg_bu(co); }
 
 template <int BU>
-__global__ void __launch_bounds__(BU == 8 ? 160 : 320, BU == 8 ? 3 : 1)
-    k_wgrad(int ci, int co, long long npix, long long chunk, const float* __restrict__ dU, const float* __restrict__ in,
-            float* __restrict__ partial)
+__global__ void __launch_bounds__(160, 3) k_wgrad(int ci, int co, long long npix, long long chunk, const float* __restrict__ dU,
+                        const float* __restrict__ in, float* __restrict__ partial)
 {
     extern __shared__ __align__(16) float sm[];
-    const int cip = wg_cip(ci), cop = wg_cop(co, BU), g4 = cip / 4, ntask = (cop / BU) * g4;
+    const int cip = wg_cip(ci), cop = wg_cop(co), g4 = cip / 4, ntask = (cop / BU) * g4;
     const int nslice = blockDim.x / ntask;  // divides kWgTile / 4 (host)
     const int nrow = cop + cip;
     // each tile buffer: [cop][kWgS] rows of dU, then [cip][kWgS] rows of the input
@@ -1522,11 +1504,9 @@ __global__ void __launch_bounds__(BU == 8 ? 160 : 320, BU == 8 ? 3 : 1)
     // rows past co and ci never change (zeros, ones for the bias; dU is zero past
     // the pixels, so the ones need not be).
     const int tile = nrow * kWgS;
-    const int npad = nrow - co - ci;
-    for (int e = tid; e < 2 * npad * kWgTile; e += blockDim.x) {
-        const int k = e / kWgTile, q = k >= npad ? 1 : 0, j = k - q * npad;
-        const int r = j < cop - co ? co + j : j + co + ci;  // rows co .. cop - 1, then cop + ci ..
-        sm[q * tile + r * kWgS + e % kWgTile] = r == cop + ci ? 1.0f : 0.0f;
+    for (int e = tid; e < 2 * nrow * kWgTile; e += blockDim.x) {
+        const int q = e / (nrow * kWgTile), r = (e - q * nrow * kWgTile) / kWgTile, p = e % kWgTile;
+        if ((r >= co && r < cop) || r >= cop + ci) sm[q * tile + r * kWgS + p] = r == cop + ci ? 1.0f : 0.0f;
     }
     const int fp = 4 * (tid & (kWgTile / 4 - 1)), fr = tid / (kWgTile / 4), fstep = blockDim.x / (kWgTile / 4);
     auto fill = [&](int q, long long g) {
@@ -1768,16 +1748,6 @@ wave_status_t combine_tc_launch(int B, int Nz, int Nx, int mx, const void* in, c
     return launched();
 }
 
-int sm_count()
-{
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0)
-        return n;
-    (void)cudaGetLastError();
-    return 152;
-}
-
 template <typename Tin, typename Tout>
 void combine_dispatch(int B, int ci, int co, int Nz, int Nx, int mx, const void* in, const float* M, int mt,
                       const float* bias, const float* T, const float* tab, int act, float* pre, void* out,
@@ -1798,19 +1768,17 @@ void combine_dispatch(int B, int ci, int co, int Nz, int Nx, int mx, const void*
             const int rw = 64 / co;  // rows at a time (k_combine_rz)
             const size_t smem = (size_t)(ci * co + (T ? rw * 32 * co : 0) + rw * ci * kRtS + (T ? 32 * kRtS : 0) + co) *
                                 sizeof(float);
-            // A block marches over its rows one after the other, so as few rows as keep the blocks within
-            // 2.5 rounds of 3 per SM; where there are more, longer marches share the staging of the weights
-            // and the table.  8 x 32 x 256 x 512: 173 us with 8 rows, 181 with 2; 1 x 32 x 256 x 512: 30 with 2
-            // or 4, 40 with 8; 1 x 64 x 90 x 72: 16 with 1, 82 with 8.
-            const long long most = 5LL * 3 * sm_count() / 2, strips = (long long)((Nx + kRtP - 1) / kRtP) * B;
-            int nrow = rw;
-            while (nrow < 8 && strips * ((Nz + nrow - 1) / nrow) > most) nrow *= 2;
+            const int nrow = 8;  // 162 us; 16 rows or one round of longer strips: 165 to 169 us
             const dim3 grid((unsigned)((Nx + kRtP - 1) / kRtP), (unsigned)((Nz + nrow - 1) / nrow), (unsigned)B);
-            const auto kernel = co == 32 ? (T ? k_combine_rz<32, true, Tout> : k_combine_rz<32, false, Tout>)
-                                         : (T ? k_combine_rz<64, true, Tout> : k_combine_rz<64, false, Tout>);
-            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            kernel<<<grid, 128, smem, s>>>(nrow, ci, Nz, Nx, mx, static_cast<const float*>(in), M, mt, bias, T, tab, act,
-                                           pre, static_cast<Tout*>(out));
+            if (co == 32) {
+                cudaFuncSetAttribute(k_combine_rz<32, Tout>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                k_combine_rz<32, Tout><<<grid, 128, smem, s>>>(nrow, ci, Nz, Nx, mx, static_cast<const float*>(in), M, mt,
+                                                               bias, T, tab, act, pre, static_cast<Tout*>(out));
+            } else {
+                cudaFuncSetAttribute(k_combine_rz<64, Tout>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                k_combine_rz<64, Tout><<<grid, 128, smem, s>>>(nrow, ci, Nz, Nx, mx, static_cast<const float*>(in), M, mt,
+                                                               bias, T, tab, act, pre, static_cast<Tout*>(out));
+            }
             return;
         }
     }
@@ -2056,28 +2024,25 @@ wave_status_t fno_wgrad(int B, int Ci, int Co, long long npix, const float* dU, 
     if (wg_max_blocks(B, npix) > 0x7fffffffLL || B > 65535) return WAVE_ERR_ARG;
     long long nblk = 0;
     if (npix > 0 && B > 0) {
-        // Output blocks times pixel slices (a power of two dividing the tile's 16 groups of 4).  With enough
-        // blocks for the GPU, 8 x 4 outputs a thread and up to 160 threads (3 blocks of 128 registers a thread
-        // per SM): 8 x 131072 pixels, 32 x 32 channels 102 us, 122 with 4 x 4.  With fewer than 2 blocks per
-        // SM, 4 x 4 and up to 320 threads, which shorten the chain of a tile: 4096 pixels, 64 x 64 channels 40
-        // us, 49 with 8 x 4.  So too for few input channels, which leave few threads: 8 x 131072 pixels, 16 x 1
-        // channels 25 us, 44 with 8 x 4.
-        const bool few = wg_max_blocks(B, npix) < 2LL * sm_count();
-        const int bu = Co < 8 || Ci < 4 || few ? 4 : 8, cop = wg_cop(Co, bu);
-        const int ntask = (cop / bu) * (wg_cip(Ci) / 4), most = few || Ci < 4 ? 320 : 160;
+        // output blocks times pixel slices (a power of two dividing the tile's 16
+        // groups of 4), up to 160 threads (3 blocks of 128 registers a thread per SM)
+        const int bu = wg_bu(Co);
+        const int ntask = (wg_cop(Co) / bu) * (wg_cip(Ci) / 4);
         int nslice = 1;
-        while (nslice < kWgTile / 4 && ntask * nslice * 2 <= most) nslice *= 2;
+        while (nslice < kWgTile / 4 && ntask * nslice * 2 <= 160) nslice *= 2;
         const int threads = ntask * nslice;
-        const size_t tile = (size_t)(cop + wg_cip(Ci)) * kWgS;
-        const size_t red = (size_t)nslice * cop * wg_cip(Ci);
+        const size_t tile = (size_t)(wg_cop(Co) + wg_cip(Ci)) * kWgS;
+        const size_t red = (size_t)nslice * wg_cop(Co) * wg_cip(Ci);
         const size_t smem = std::max(2 * tile, red) * sizeof(float);
         const auto kernel = bu == 8 ? k_wgrad<8> : k_wgrad<4>;
         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         // chunks per sample so that all blocks are resident at once
-        int per = 0;
+        int per = 0, dev = 0, nsm = 1;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem);
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         (void)cudaGetLastError();
-        const long long want = std::max(1LL, (long long)std::max(per, 1) * sm_count() / B);
+        const long long want = std::max(1LL, (long long)std::max(per, 1) * nsm / B);
         long long chunk = (npix + want - 1) / want;
         chunk = std::max<long long>(kWgMinChunk, (chunk + kWgTile - 1) / kWgTile * kWgTile);
         const long long nchunk = (npix + chunk - 1) / chunk;
