@@ -794,18 +794,18 @@ __device__ __forceinline__ void cp_async_wait_stages() { asm volatile("cp.async.
 // outputs 8 oq .. 8 oq + 7 at pixels 4 pq .. + 3 and 64 + 4 pq .. + 3: per k, four
 // 16-byte shared-memory loads feed 64 products (32 FFMA2), so loads and FMAs take
 // the same time; 4 x 8 blocks were bound by their loads (l1tex 69 % busy, 160 us
-// per launch at 8 x 32 x 256 x 512).  The same k order and fmaf sequence as
-// k_combine (bitwise the same outputs).
-template <int CO, typename Tout>
-__global__ void __launch_bounds__(128, 3) k_combine_rz(int nrow, int ci, int Nz, int Nx, int mx, const float* __restrict__ in,
-                                                       const float* __restrict__ M, int mtrans,
-                                                       const float* __restrict__ bias, const float* __restrict__ T,
-                                                       const float* __restrict__ tab, int act, float* __restrict__ pre,
-                                                       Tout* __restrict__ out)
+// per launch at 8 x 32 x 256 x 512).  Without the spectral part 4 blocks fit an SM (91
+// us at that size, 96 with 3).  The same k order and fmaf sequence as k_combine
+// (bitwise the same outputs).
+template <int CO, bool SPEC, typename Tout>
+__global__ void __launch_bounds__(128, SPEC ? 3 : 4)
+    k_combine_rz(int nrow, int ci, int Nz, int Nx, int mx, const float* __restrict__ in, const float* __restrict__ M,
+                 int mtrans, const float* __restrict__ bias, const float* __restrict__ T, const float* __restrict__ tab,
+                 int act, float* __restrict__ pre, Tout* __restrict__ out)
 {
     extern __shared__ __align__(16) float sm[];
     constexpr int NT = 128, RW = NT / (CO * 2), TPT = RW * 32 * CO / NT;  // coefficients per thread (16)
-    const bool spec = T != nullptr;
+    const bool spec = SPEC && T != nullptr;  // (a test at run time: without it the compiler schedules the sums 2 % slower)
     float* sW = sm;                                   // [ci][CO]
     float* sT = sW + ci * CO;                         // [RW][32][CO] (spec)
     float* sX = sT + (spec ? RW * 32 * CO : 0);       // [RW][ci][kRtS]
@@ -1748,6 +1748,16 @@ wave_status_t combine_tc_launch(int B, int Nz, int Nx, int mx, const void* in, c
     return launched();
 }
 
+int sm_count()
+{
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0)
+        return n;
+    (void)cudaGetLastError();
+    return 152;
+}
+
 template <typename Tin, typename Tout>
 void combine_dispatch(int B, int ci, int co, int Nz, int Nx, int mx, const void* in, const float* M, int mt,
                       const float* bias, const float* T, const float* tab, int act, float* pre, void* out,
@@ -1768,17 +1778,19 @@ void combine_dispatch(int B, int ci, int co, int Nz, int Nx, int mx, const void*
             const int rw = 64 / co;  // rows at a time (k_combine_rz)
             const size_t smem = (size_t)(ci * co + (T ? rw * 32 * co : 0) + rw * ci * kRtS + (T ? 32 * kRtS : 0) + co) *
                                 sizeof(float);
-            const int nrow = 8;  // 162 us; 16 rows or one round of longer strips: 165 to 169 us
+            // A block marches over its rows one after the other, so as few rows as keep the blocks within
+            // 2.5 rounds of 3 per SM; where there are more, longer marches share the staging of the weights
+            // and the table.  8 x 32 x 256 x 512: 173 us with 8 rows, 181 with 2; 1 x 32 x 256 x 512: 30 with 2
+            // or 4, 40 with 8; 1 x 64 x 90 x 72: 16 with 1, 82 with 8.
+            const long long most = 5LL * 3 * sm_count() / 2, strips = (long long)((Nx + kRtP - 1) / kRtP) * B;
+            int nrow = rw;
+            while (nrow < 8 && strips * ((Nz + nrow - 1) / nrow) > most) nrow *= 2;
             const dim3 grid((unsigned)((Nx + kRtP - 1) / kRtP), (unsigned)((Nz + nrow - 1) / nrow), (unsigned)B);
-            if (co == 32) {
-                cudaFuncSetAttribute(k_combine_rz<32, Tout>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                k_combine_rz<32, Tout><<<grid, 128, smem, s>>>(nrow, ci, Nz, Nx, mx, static_cast<const float*>(in), M, mt,
-                                                               bias, T, tab, act, pre, static_cast<Tout*>(out));
-            } else {
-                cudaFuncSetAttribute(k_combine_rz<64, Tout>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                k_combine_rz<64, Tout><<<grid, 128, smem, s>>>(nrow, ci, Nz, Nx, mx, static_cast<const float*>(in), M, mt,
-                                                               bias, T, tab, act, pre, static_cast<Tout*>(out));
-            }
+            const auto kernel = co == 32 ? (T ? k_combine_rz<32, true, Tout> : k_combine_rz<32, false, Tout>)
+                                         : (T ? k_combine_rz<64, true, Tout> : k_combine_rz<64, false, Tout>);
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            kernel<<<grid, 128, smem, s>>>(nrow, ci, Nz, Nx, mx, static_cast<const float*>(in), M, mt, bias, T, tab, act,
+                                           pre, static_cast<Tout*>(out));
             return;
         }
     }
