@@ -1472,16 +1472,15 @@ inline long long wg_max_blocks(int B, long long npix) { return B * ((npix + kWgM
 // FMA: with BU = 8, 12 16-byte loads and 64 FFMA2 per 128 products, where 4 x 4
 // blocks of scalar FMAs took 16 loads and 128 (shared-memory bound).
 constexpr int kWgS = kWgTile + 4;
-// outputs per thread along o: 8, or 4 for few output channels
-__host__ __device__ inline int wg_bu(int co) { return co >= 8 ? 8 : 4; }
-__host__ __device__ inline int wg_cop(int co) { return (co + wg_bu(co) - 1) / wg_bu(co) * wg_bu(co); }
+__host__ __device__ inline int wg_cop(int co, int bu) { return (co + bu - 1) / bu * bu; }
 
 template <int BU>
-__global__ void __launch_bounds__(160, 3) k_wgrad(int ci, int co, long long npix, long long chunk, const float* __restrict__ dU,
-                        const float* __restrict__ in, float* __restrict__ partial)
+__global__ void __launch_bounds__(BU == 8 ? 160 : 320, BU == 8 ? 3 : 1)
+    k_wgrad(int ci, int co, long long npix, long long chunk, const float* __restrict__ dU, const float* __restrict__ in,
+            float* __restrict__ partial)
 {
     extern __shared__ __align__(16) float sm[];
-    const int cip = wg_cip(ci), cop = wg_cop(co), g4 = cip / 4, ntask = (cop / BU) * g4;
+    const int cip = wg_cip(ci), cop = wg_cop(co, BU), g4 = cip / 4, ntask = (cop / BU) * g4;
     const int nslice = blockDim.x / ntask;  // divides kWgTile / 4 (host)
     const int nrow = cop + cip;
     // each tile buffer: [cop][kWgS] rows of dU, then [cip][kWgS] rows of the input
@@ -1504,9 +1503,11 @@ __global__ void __launch_bounds__(160, 3) k_wgrad(int ci, int co, long long npix
     // rows past co and ci never change (zeros, ones for the bias; dU is zero past
     // the pixels, so the ones need not be).
     const int tile = nrow * kWgS;
-    for (int e = tid; e < 2 * nrow * kWgTile; e += blockDim.x) {
-        const int q = e / (nrow * kWgTile), r = (e - q * nrow * kWgTile) / kWgTile, p = e % kWgTile;
-        if ((r >= co && r < cop) || r >= cop + ci) sm[q * tile + r * kWgS + p] = r == cop + ci ? 1.0f : 0.0f;
+    const int npad = nrow - co - ci;
+    for (int e = tid; e < 2 * npad * kWgTile; e += blockDim.x) {
+        const int k = e / kWgTile, q = k >= npad ? 1 : 0, j = k - q * npad;
+        const int r = j < cop - co ? co + j : j + co + ci;  // rows co .. cop - 1, then cop + ci ..
+        sm[q * tile + r * kWgS + e % kWgTile] = r == cop + ci ? 1.0f : 0.0f;
     }
     const int fp = 4 * (tid & (kWgTile / 4 - 1)), fr = tid / (kWgTile / 4), fstep = blockDim.x / (kWgTile / 4);
     auto fill = [&](int q, long long g) {
@@ -2036,25 +2037,28 @@ wave_status_t fno_wgrad(int B, int Ci, int Co, long long npix, const float* dU, 
     if (wg_max_blocks(B, npix) > 0x7fffffffLL || B > 65535) return WAVE_ERR_ARG;
     long long nblk = 0;
     if (npix > 0 && B > 0) {
-        // output blocks times pixel slices (a power of two dividing the tile's 16
-        // groups of 4), up to 160 threads (3 blocks of 128 registers a thread per SM)
-        const int bu = wg_bu(Co);
-        const int ntask = (wg_cop(Co) / bu) * (wg_cip(Ci) / 4);
+        // Output blocks times pixel slices (a power of two dividing the tile's 16 groups of 4).  With enough
+        // blocks for the GPU, 8 x 4 outputs a thread and up to 160 threads (3 blocks of 128 registers a thread
+        // per SM): 8 x 131072 pixels, 32 x 32 channels 102 us, 122 with 4 x 4.  With fewer than 2 blocks per
+        // SM, 4 x 4 and up to 320 threads, which shorten the chain of a tile: 4096 pixels, 64 x 64 channels 40
+        // us, 49 with 8 x 4.  So too for few input channels, which leave few threads: 8 x 131072 pixels, 16 x 1
+        // channels 25 us, 44 with 8 x 4.
+        const bool few = wg_max_blocks(B, npix) < 2LL * sm_count();
+        const int bu = Co < 8 || Ci < 4 || few ? 4 : 8, cop = wg_cop(Co, bu);
+        const int ntask = (cop / bu) * (wg_cip(Ci) / 4), most = few || Ci < 4 ? 320 : 160;
         int nslice = 1;
-        while (nslice < kWgTile / 4 && ntask * nslice * 2 <= 160) nslice *= 2;
+        while (nslice < kWgTile / 4 && ntask * nslice * 2 <= most) nslice *= 2;
         const int threads = ntask * nslice;
-        const size_t tile = (size_t)(wg_cop(Co) + wg_cip(Ci)) * kWgS;
-        const size_t red = (size_t)nslice * wg_cop(Co) * wg_cip(Ci);
+        const size_t tile = (size_t)(cop + wg_cip(Ci)) * kWgS;
+        const size_t red = (size_t)nslice * cop * wg_cip(Ci);
         const size_t smem = std::max(2 * tile, red) * sizeof(float);
         const auto kernel = bu == 8 ? k_wgrad<8> : k_wgrad<4>;
         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         // chunks per sample so that all blocks are resident at once
-        int per = 0, dev = 0, nsm = 1;
+        int per = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem);
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         (void)cudaGetLastError();
-        const long long want = std::max(1LL, (long long)std::max(per, 1) * nsm / B);
+        const long long want = std::max(1LL, (long long)std::max(per, 1) * sm_count() / B);
         long long chunk = (npix + want - 1) / want;
         chunk = std::max<long long>(kWgMinChunk, (chunk + kWgTile - 1) / kWgTile * kWgTile);
         const long long nchunk = (npix + chunk - 1) / chunk;

@@ -1,11 +1,13 @@
-"""FNO channel mixes with 1 to 8 rows per block, by how much there is to do.  Small maps
-must not pay for what large ones gain."""
+"""FNO kernels whose launch depends on how much there is to do: channel mixes with 1 to 8
+rows per block, weight gradients with either block height.  Small maps must not pay for
+what large ones gain."""
 import pytest
 import torch
 
 from paper_2304_05592_gb300 import fno
 
 pytestmark = pytest.mark.gpu
+EPS = 2.0 ** -24
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -72,3 +74,30 @@ def test_a_small_channel_mix_takes_a_fraction_of_a_larger_one(co, spec):
         return _us(lambda: fno.fno_combine(v, M, co, bias=b, T=T, table=tab, mx=16, act=fno.ACT_GELU, out=out))
 
     assert t(1) < 0.75 * t(8)  # (equal with 8 rows per block for both)
+
+
+def _wgrad(B, ci, co, npix):
+    dU, v = _rand((B, co, 1, npix), 10), _rand((B, ci, 1, npix), 11)
+    dM, db = torch.empty((co, ci), device="cuda"), torch.empty((co,), device="cuda")
+    work = torch.empty(max(1, fno.fno_wgrad_work_floats(B, ci, co, npix)), device="cuda")
+    return dU, v, dM, db, work
+
+
+# either side of 2 x 152 blocks of 512 pixels, of 8 outputs and of 4 inputs
+@pytest.mark.parametrize("B,npix", [(1, 1), (2, 130), (1, 303 * 512), (1, 304 * 512 + 3), (5, 40000)])
+@pytest.mark.parametrize("ci,co", [(1, 16), (3, 64), (4, 8), (4, 7), (33, 20), (64, 64)])
+def test_weight_gradients_either_side_of_the_rule(B, npix, ci, co):
+    dU, v, dM, db, work = _wgrad(B, ci, co, npix)
+    fno.fno_wgrad(dU, v, dM, db, work)
+    d, x = dU.double().reshape(B, co, -1), v.double().reshape(B, ci, -1)
+    for got, ref, mag in ((dM, torch.einsum("bop,bip->oi", d, x), torch.einsum("bop,bip->oi", d.abs(), x.abs())),
+                          (db, d.sum((0, 2)), d.abs().sum((0, 2)))):
+        assert not bool(((got.double() - ref).abs() > (B * npix + 2) * EPS * mag + 1e-30).any())
+
+
+def test_one_input_channel_takes_no_longer_than_sixteen():
+    def t(ci):
+        dU, v, dM, db, work = _wgrad(1, ci, 16, 4096)
+        return _us(lambda: fno.fno_wgrad(dU, v, dM, db, work))
+
+    assert t(1) <= t(16)
