@@ -261,6 +261,13 @@ __device__ __forceinline__ void cp_async8(void* dst, const void* src, bool ok)
                  : "memory");
 }
 
+__device__ __forceinline__ void cp_async16z(void* dst, const void* src, bool ok)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(ok ? 16 : 0)
+                 : "memory");
+}
+
 // out[b][a][kx] = sum_z in[b][z][kx] conj(E[z][a]); CTA per (b, 16 values of a).
 // Thread (h, q, kx) computes outputs (a0 + 4 q .. a0 + 4 q + 3, kx) over quarter h
 // of every 64-row chunk of z, so each in[z][kx] read from shared memory feeds
@@ -272,14 +279,26 @@ __global__ void __launch_bounds__(256) k_dft_z(int Nz, int KZ, int mx, const flo
     __shared__ float2 red[3][16][16];
     const int b = blockIdx.x, a0 = blockIdx.y * 16, tid = threadIdx.x;
     const int kx = tid & 15, q = (tid >> 4) & 3, h = tid >> 6;
-    // rows z0 .. z0 + 63 of the input and the table into buffer w (8-byte copies, zeros outside)
+    // rows z0 .. z0 + 63 of the input and the table into buffer w, zeros outside: two modes per copy where
+    // rows begin at 16 bytes (KZ = 2 mz is even), else one
+    const bool pairs = (mx & 1) == 0 && ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(tz)) & 15) == 0;
     auto fill = [&](int z0, int w) {
+        if (pairs) {
 #pragma unroll
-        for (int e = tid; e < 64 * 16; e += 256) {
-            const int zz = e >> 4, k = e & 15, z = z0 + zz;
-            const bool vi = z < Nz && k < mx, ve = z < Nz && a0 + k < KZ;
-            cp_async8(&si[w][zz][k], vi ? in + ((size_t)b * Nz + z) * mx + k : in, vi);
-            cp_async8(&se[w][zz][k], ve ? tz + (size_t)z * KZ + a0 + k : tz, ve);
+            for (int e = tid; e < 64 * 8; e += 256) {
+                const int zz = e >> 3, k = 2 * (e & 7), z = z0 + zz;
+                const bool vi = z < Nz && k < mx, ve = z < Nz && a0 + k < KZ;
+                cp_async16z(&si[w][zz][k], vi ? in + ((size_t)b * Nz + z) * mx + k : in, vi);
+                cp_async16z(&se[w][zz][k], ve ? tz + (size_t)z * KZ + a0 + k : tz, ve);
+            }
+        } else {
+#pragma unroll
+            for (int e = tid; e < 64 * 16; e += 256) {
+                const int zz = e >> 4, k = e & 15, z = z0 + zz;
+                const bool vi = z < Nz && k < mx, ve = z < Nz && a0 + k < KZ;
+                cp_async8(&si[w][zz][k], vi ? in + ((size_t)b * Nz + z) * mx + k : in, vi);
+                cp_async8(&se[w][zz][k], ve ? tz + (size_t)z * KZ + a0 + k : tz, ve);
+            }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };

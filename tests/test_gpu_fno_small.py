@@ -1,6 +1,6 @@
 """FNO kernels whose launch depends on how much there is to do: channel mixes with 1 to 8
-rows per block, weight gradients with either block height.  Small maps must not pay for
-what large ones gain."""
+rows per block, weight gradients with either block height, z transforms by pairs of
+modes and singly.  Small maps must not pay for what large ones gain."""
 import pytest
 import torch
 
@@ -101,3 +101,19 @@ def test_one_input_channel_takes_no_longer_than_sixteen():
         return _us(lambda: fno.fno_wgrad(dU, v, dM, db, work))
 
     assert t(1) <= t(16)
+
+
+@pytest.mark.parametrize("mx", [1, 7, 8, 15, 16])
+@pytest.mark.parametrize("Nz,mz", [(31, 3), (64, 16), (131, 9)])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_z_transform_by_pairs_and_singly(mx, Nz, mz, shift):
+    """shift: inputs one complex number past a 16-byte boundary."""
+    nb = 3
+    x, tz = (_rand((n + 2 * shift,), 8 + n)[2 * shift:].view(*s, 2) for n, s in
+             ((nb * Nz * mx * 2, (nb, Nz, mx)), (Nz * 2 * mz * 2, (Nz, 2 * mz))))
+    assert x.data_ptr() % 16 == 8 * shift
+    got = torch.view_as_complex(fno.fno_dft_z(x, nb, Nz, mz, mx, tz).double())
+    X, E = torch.view_as_complex(x.double()), torch.view_as_complex(tz.double()).conj()
+    mag = torch.einsum("bzk,za->bak", X.abs(), E.abs())
+    err = (got.view(nb, 2 * mz, mx) - torch.einsum("bzk,za->bak", X, E)).abs()
+    assert bool((err <= 4 * (Nz + 2) * EPS * mag).all())
