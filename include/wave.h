@@ -356,7 +356,10 @@ wave_status_t wave_profile_stop(double* fwd_ms, long long* fwd_n, double* adj_ms
  * forward step, 1 the 2D adjoint step, 2 the 3D step (forward and adjoint);
  * variant in [0, wave_variant_count(which)) or -1 for the library default.
  * 2D variants: direct loads, TMA pipeline, shot groups (cp.async or TMA fed),
- * z-march, persistent items, with different tile shapes; 3D variants: a
+ * z-march, persistent items, z-window, with different tile shapes, and last the
+ * on-chip loop, which makes many time steps per launch (a problem it cannot
+ * take runs by shot groups); the default takes the loop or shot groups of 1, 2
+ * or 4, by an estimate of their times.  3D variants: a
  * z-march with a shared-memory halo plane (0) and TMA plane rings with
  * different tile heights and z chunks.  All variants of a step compute the
  * same shot records bit for bit (one arithmetic order); gradients agree to

@@ -44,7 +44,7 @@ struct DevTaps {
 //   forward  : W0 W1
 //   adjoint  : A0 A1
 //   gradient : W0 W1 A0 A1 G Z S(0).cur S(0).prev ... [FP32 store rows 0..nt-1]
-//   Born     : W0 W1 W2 (background levels) A0 A1 (scattered levels)
+//   Born     : W0 W1, in 3D W2 (background levels) A0 A1 (scattered levels)
 // W = forward levels, A = adjoint levels, G = per-shot gradient accumulators,
 // Z = a zero batch (the state before the first step), S(k) = checkpoint slot k.
 // The first 256 bytes of every workspace: the device error word of the last

@@ -653,7 +653,15 @@ struct ChipShape {
 // The register file (16384 per scheduler) bounds the block: 4 warps per
 // scheduler leave 128 registers a thread, 5 leave 96, 6 leave 80.  A thread
 // holds 4 RB model values (with imaging 4 RB gradient values instead, the model
-// in shared memory), the 36-value z window and about 35 others.
+// in shared memory), the 36-value z window and about 35 others.  What exceeds the
+// cap spills (bytes of stores / loads per thread): with imaging 8 rows 136 / 156, 7
+// rows 72 / 116 (FP32 level; 68 / 88 BF16), 6 rows 60 / 68; without, 10 rows 44 / 44, 4
+// rows 44 / 52 and 2 rows 48 / 52 at their 5 and 6 warps, 5 to 8 rows 28 at most.  The cap
+// is the shape's, also for a plan of fewer threads (448 of 512 for 592 x 336 on 16 CTAs).
+// Of 260 random problems (30 to 700 x 30 to 400 points, sponges of 0 to 40 cells, 1 to 24
+// shots) forward steps took 2 rows in 210, 3 in 15, 4 in 13, and 5 to 10 in 2 to 4 each,
+// launches kept 5; the shapes of 4, 5 and 6 rows that form the factors were
+// not taken forward, the one of 4 rows not at all.
 template <int RB, int NF, int NA, bool EPS>
 constexpr ChipShape shape()
 {
