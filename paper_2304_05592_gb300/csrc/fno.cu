@@ -1884,8 +1884,8 @@ wave_status_t fno_dft_x(long long rows, int Nx, int mx, const void* in, int in_b
     else if (mx == 16 && (Nx & 3) == 0 &&
              ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(table) | reinterpret_cast<uintptr_t>(out)) &
               15) == 0) {
-        // (256-row CTAs need 4 per SM to hide their latency: 155648 rows)
-        if (rows >= 256LL * 4 * 152)
+        // (256-row CTAs need 4 per SM to hide their latency: 155648 rows on 152 SMs)
+        if (rows >= 256LL * 4 * sm_count())
             k_dft_x8<8><<<(unsigned)((rows + 255) / 256), 128, 0, s>>>(rows, Nx, static_cast<const float*>(in), table, out);
         else
             k_dft_x8<4><<<(unsigned)((rows + 127) / 128), 128, 0, s>>>(rows, Nx, static_cast<const float*>(in), table, out);
