@@ -1493,7 +1493,7 @@ inline long long wg_max_blocks(int B, long long npix) { return B * ((npix + kWgM
 constexpr int kWgS = kWgTile + 4;
 __host__ __device__ inline int wg_cop(int co, int bu) { return (co + bu - 1) / bu * bu; }
 
-template <int BU>
+template <int BU, bool VEC>  // VEC: rows begin at 16 bytes
 __global__ void __launch_bounds__(BU == 8 ? 160 : 320, BU == 8 ? 3 : 1)
     k_wgrad(int ci, int co, long long npix, long long chunk, const float* __restrict__ dU, const float* __restrict__ in,
             float* __restrict__ partial)
@@ -1509,8 +1509,6 @@ __global__ void __launch_bounds__(BU == 8 ? 160 : 320, BU == 8 ? 3 : 1)
     const long long p0 = (long long)blockIdx.x * chunk, p1 = min(p0 + chunk, npix);
     const float* dUb = dU + (size_t)b * co * npix;
     const float* inb = in + (size_t)b * ci * npix;
-    const bool vec = (npix & 3) == 0 && (reinterpret_cast<uintptr_t>(dU) & 15) == 0 &&
-                     (reinterpret_cast<uintptr_t>(in) & 15) == 0;
     float2 acc[BU][4];  // sums over even and odd pixels
 #pragma unroll
     for (int u = 0; u < BU; ++u)
@@ -1537,14 +1535,24 @@ __global__ void __launch_bounds__(BU == 8 ? 160 : 320, BU == 8 ? 3 : 1)
                 const int rows = part ? ci : co;
                 const float* src = (part ? inb : dUb) + (size_t)fr * npix + g + fp;
                 float* d = dst + ((part ? cop : 0) + fr) * kWgS;
-                if (vec) {
+                if (VEC) {
                     const int bytes = 4 * max(0, min(4, n));  // zero fill past the pixels
                     for (int r = fr; r < rows; r += fstep, src += (size_t)fstep * npix, d += fstep * kWgS)
                         cp_async16(su32(d), bytes ? src : dUb, bytes);
                 } else {
-                    for (int r = fr; r < rows; r += fstep, src += (size_t)fstep * npix, d += fstep * kWgS)
-                        *reinterpret_cast<float4*>(d) = make_float4(n > 0 ? src[0] : 0.0f, n > 1 ? src[1] : 0.0f,
-                                                                    n > 2 ? src[2] : 0.0f, n > 3 ? src[3] : 0.0f);
+                    for (int r = fr; r < rows; r += 4 * fstep, src += (size_t)(4 * fstep) * npix, d += 4 * fstep * kWgS) {
+                        float v[4][4];  // 4 rows' loads in flight before the first is stored
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+                                v[k][e] = r + k * fstep < rows && n > e ? src[(size_t)(k * fstep) * npix + e] : 0.0f;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            if (r + k * fstep < rows)
+                                *reinterpret_cast<float4*>(d + k * fstep * kWgS) =
+                                    make_float4(v[k][0], v[k][1], v[k][2], v[k][3]);
+                    }
                 }
             }
         }
@@ -2071,7 +2079,9 @@ wave_status_t fno_wgrad(int B, int Ci, int Co, long long npix, const float* dU, 
         const size_t tile = (size_t)(cop + wg_cip(Ci)) * kWgS;
         const size_t red = (size_t)nslice * cop * wg_cip(Ci);
         const size_t smem = std::max(2 * tile, red) * sizeof(float);
-        const auto kernel = bu == 8 ? k_wgrad<8> : k_wgrad<4>;
+        const bool vec = (npix & 3) == 0 && ((reinterpret_cast<uintptr_t>(dU) | reinterpret_cast<uintptr_t>(in)) & 15) == 0;
+        const auto kernel = bu == 8 ? (vec ? k_wgrad<8, true> : k_wgrad<8, false>)
+                                    : (vec ? k_wgrad<4, true> : k_wgrad<4, false>);
         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         // chunks per sample so that all blocks are resident at once
         int per = 0;

@@ -117,3 +117,13 @@ def test_z_transform_by_pairs_and_singly(mx, Nz, mz, shift):
     mag = torch.einsum("bzk,za->bak", X.abs(), E.abs())
     err = (got.view(nb, 2 * mz, mx) - torch.einsum("bzk,za->bak", X, E)).abs()
     assert bool((err <= 4 * (Nz + 2) * EPS * mag).all())
+
+
+@pytest.mark.parametrize("ci,co", [(43, 64), (43, 7)])
+def test_odd_maps_take_little_more_than_even_ones(ci, co):
+    """Rows that do not begin at 16 bytes are loaded pixel by pixel, with enough loads in flight."""
+    def t(npix):
+        dU, v, dM, db, work = _wgrad(3, ci, co, npix)
+        return _us(lambda: fno.fno_wgrad(dU, v, dM, db, work))
+
+    assert t(131071) < 1.6 * t(131072)
