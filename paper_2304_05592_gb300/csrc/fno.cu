@@ -2066,8 +2066,8 @@ wave_status_t fno_wgrad(int B, int Ci, int Co, long long npix, const float* dU, 
     if (npix > 0 && B > 0) {
         // Output blocks times pixel slices (a power of two dividing the tile's 16 groups of 4).  With enough
         // blocks for the GPU, 8 x 4 outputs a thread and up to 160 threads (3 blocks of 128 registers a thread
-        // per SM): 8 x 131072 pixels, 32 x 32 channels 102 us, 122 with 4 x 4.  With fewer than 2 blocks per
-        // SM, 4 x 4 and up to 320 threads, which shorten the chain of a tile: 4096 pixels, 64 x 64 channels 40
+        // per SM): 8 x 131072 pixels, 32 x 32 channels 101 us, 122 with 4 x 4.  With fewer than 2 blocks per
+        // SM, 4 x 4 and up to 320 threads, which shorten the chain of a tile: 4096 pixels, 64 x 64 channels 34
         // us, 49 with 8 x 4.  So too for few input channels, which leave few threads: 8 x 131072 pixels, 16 x 1
         // channels 25 us, 44 with 8 x 4.
         const bool few = wg_max_blocks(B, npix) < 2LL * sm_count();

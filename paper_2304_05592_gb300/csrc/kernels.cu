@@ -28,14 +28,6 @@ __device__ __forceinline__ float leap(float c, float um, float lap, float kap, f
     return num * rcp_sponge(1.0f + eps);
 }
 
-// The same update with an extra source term subtracted before the damping
-// factor (the Born secondary source); src = 0 gives exactly leap().
-__device__ __forceinline__ float leap_src(float c, float um, float lap, float kap, float eps, float src)
-{
-    float num = fmaf(kap, lap, fmaf(eps, um, 2.0f * c - um)) - src;
-    return num * rcp_sponge(1.0f + eps);
-}
-
 // Born secondary source of four points: dmv .* (u^{n+1} - 2 u^n + u^{n-1}),
 // with dmv = dm v^2 (it enters the update as kap * lap - src).
 __device__ __forceinline__ void born_source(const StepArgs& a, long long so, long long off, float* src)
