@@ -20,14 +20,6 @@
 namespace wave {
 
 
-// One leapfrog update in Courant units:
-//   (1+eps) u+ = 2u - (1-eps) u- + kap * lap,  kap = (v dt/h)^2, eps = eta dt v^2 / 2.
-__device__ __forceinline__ float leap(float c, float um, float lap, float kap, float eps)
-{
-    float num = fmaf(kap, lap, fmaf(eps, um, 2.0f * c - um));
-    return num * rcp_sponge(1.0f + eps);
-}
-
 // Born secondary source of four points: dmv .* (u^{n+1} - 2 u^n + u^{n-1}),
 // with dmv = dm v^2 (it enters the update as kap * lap - src).
 __device__ __forceinline__ void born_source(const StepArgs& a, long long so, long long off, float* src)
